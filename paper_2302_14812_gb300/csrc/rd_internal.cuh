@@ -133,7 +133,7 @@ __device__ __forceinline__ void item_coords(unsigned idx, const DepositParams& P
 
 constexpr int kDepositThreads = 256;   // FP64 kernel: one cell per thread
 #ifndef RD_MIXED_MINBLOCKS
-#define RD_MIXED_MINBLOCKS (RD_MIXED_CELLS >= 4 ? 6 : 5)
+#define RD_MIXED_MINBLOCKS (RD_MIXED_CELLS >= 4 ? 6 : 4)
 #endif
 #ifndef RD_MIXED_CELLS
 #define RD_MIXED_CELLS 2

@@ -46,11 +46,28 @@ struct Cells {
     float gpp[6][NC];               // quadratic interpolation: scaled field two samples back ...
     float hp[NC];                   // ... and the previous interval's length (units of dt)
     int bo[NC];                     // row * n_bins + bin being filled (bin may lie outside the window)
-    int rb[NC];                     // row * n_bins (row = the cell's index inside the CTA's block)
-    bool live[NC];                  // some arrival of the chunk falls inside the window
-    int below[NC];                  // intervals whose start lies before the window (clip tracking only)
-    int above[NC];                  // intervals whose end lies after the window (clip tracking only)
 };
+
+// What a cell needs only at the ends of its chunk, kept in shared memory ([word][thread]) so that the
+// walk's registers hold nothing but its running state.
+enum { kBoEnd, kFEnd, kBelow, kAbove, kColdWords };
+template <int NC, int NT>
+struct Cold {
+    float (*w)[NT];                 // [NC * kColdWords][NT]
+    // row * n_bins + bin, and time inside that bin, of the chunk's last arrival (exact FP64 anchor)
+    __device__ __forceinline__ int bo_end(int j) const { return __float_as_int(w[j * kColdWords + kBoEnd][threadIdx.x]); }
+    __device__ __forceinline__ float f_end(int j) const { return w[j * kColdWords + kFEnd][threadIdx.x]; }
+    // intervals whose start lies before / whose end lies after the window; below = -1: a cell without
+    // arrivals in the window
+    __device__ __forceinline__ int below(int j) const { return __float_as_int(w[j * kColdWords + kBelow][threadIdx.x]); }
+    __device__ __forceinline__ int above(int j) const { return __float_as_int(w[j * kColdWords + kAbove][threadIdx.x]); }
+    __device__ __forceinline__ void set(int j, int word, int v) const { w[j * kColdWords + word][threadIdx.x] = __int_as_float(v); }
+    __device__ __forceinline__ void set(int j, int word, float v) const { w[j * kColdWords + word][threadIdx.x] = v; }
+};
+
+// Offset of cell row j's first bin: row * n_bins (row = the cell's index inside the CTA's block).
+template <int NT>
+__device__ __forceinline__ int row_base(int j, int n_bins) { return (j * NT + (int)threadIdx.x) * n_bins; }
 
 #ifndef RD_CHECK
 #define RD_CHECK 0   // 1: the walk's unguarded reductions check their bin (a checked build, for tests)
@@ -209,20 +226,20 @@ __device__ __forceinline__ void field_at_ff(const RecS& r, float nx, float ny, f
 // Interval of cell j that passes two or more bin edges (rare): flush the bin being filled and the
 // whole bins inside the interval, leaving the state one edge short so that the common path below
 // finishes the step (it flushes the last whole bin and starts the next).
-template <int NC, bool TRACK, bool FF>
-__device__ __forceinline__ void multi_edges(Cells<NC>& c, int j, const Field& o, const Consts& C, float& fn, int k,
-                                            int k_begin, int k_end)
+template <int NC, int NT, bool TRACK, bool FF>
+__device__ __forceinline__ void multi_edges(Cells<NC>& c, const Cold<NC, NT>& cold, int j, const Field& o,
+                                            const Consts& C, float& fn, int k, int k_begin, int k_end)
 {
     const float f = fn;
     if (!(f >= 2.f * C.W)) return;
-    const int b0 = c.bo[j] - c.rb[j];
+    const int rb = row_base<NT>(j, C.n_bins), b0 = c.bo[j] - rb;
     const int m = (int)fminf(floorf(f * C.invW), 16777216.f);      // edges passed, >= 2
     flush_acc<NC, FF>(C, c, j, b0, c.bo[j]);
     const float fs = C.W * o.S, fb = fs * o.rinv;
     // whole bins b0+1 .. b0+m-2 now; bin b0+m-1 is left in the accumulator for the common path
     const int lo = max(b0 + 1, 0), hi = min(b0 + m - 2, C.n_bins - 1);
     for (int b = lo; b <= hi; ++b)
-        flush(C, b, c.rb[j] + b, o.E[0] * fs, o.E[1] * fs, o.E[2] * fs, o.B[0] * fb, o.B[1] * fb, o.B[2] * fb);
+        flush(C, b, rb + b, o.E[0] * fs, o.E[1] * fs, o.E[2] * fs, o.B[0] * fb, o.B[1] * fb, o.B[2] * fb);
 #pragma unroll
     for (int i = 0; i < 3; ++i) {
         c.acc[i][j] = o.E[i] * fs;
@@ -231,8 +248,8 @@ __device__ __forceinline__ void multi_edges(Cells<NC>& c, int j, const Field& o,
     c.bo[j] += m - 1;
     fn = fminf(fmaxf(fmaf(-(float)(m - 1), C.W, f), C.W), C.W * 1.99999988f);
     if (TRACK) {
-        if (b0 < 0 && b0 + m - 1 >= 0) c.below[j] = k - k_begin + 1;
-        if (b0 < C.n_bins && b0 + m - 1 >= C.n_bins) c.above[j] = k_end - k + 1;
+        if (b0 < 0 && b0 + m - 1 >= 0) cold.set(j, kBelow, k - k_begin + 1);
+        if (b0 < C.n_bins && b0 + m - 1 >= C.n_bins) cold.set(j, kAbove, k_end - k + 1);
     }
 }
 
@@ -260,15 +277,16 @@ __device__ __forceinline__ void scaled_field(const Field& o, float* G)
 // s^2 (s/3 - L/2): int_0^s t (t - L) dt
 __device__ __forceinline__ float qcube(float s, float L) { return (s * s) * fmaf(s, 1.f / 3.f, -0.5f * L); }
 
-template <int NC, bool TRACK, bool FF, bool QUAD>
-__device__ __forceinline__ void multi_edges_lin(Cells<NC>& c, int j, const float* G, const float* D2, float L,
-                                                float inv2L, const Consts& C, float& fn, int k, int k_begin, int k_end)
+template <int NC, int NT, bool TRACK, bool FF, bool QUAD>
+__device__ __forceinline__ void multi_edges_lin(Cells<NC>& c, const Cold<NC, NT>& cold, int j, const float* G,
+                                                const float* D2, float L, float inv2L, const Consts& C, float& fn,
+                                                int k, int k_begin, int k_end)
 {
     constexpr int NF = FF ? 3 : 6;                                  // carried field components
     const float f = fn;
     if (!(f >= 2.f * C.W)) return;
     const float f0 = c.f[j];
-    const int b0 = c.bo[j] - c.rb[j];
+    const int b0 = c.bo[j] - row_base<NT>(j, C.n_bins);
     const int m = (int)fminf(floorf(f * C.invW), 16777216.f);      // edges passed, >= 2
     flush_acc<NC, FF>(C, c, j, b0, c.bo[j]);
     // whole bins b0+i, i = 1..m-1, cover [i W, (i+1) W] from the start of bin b0
@@ -301,8 +319,8 @@ __device__ __forceinline__ void multi_edges_lin(Cells<NC>& c, int j, const float
     c.bo[j] += m;
     fn = fminf(fmaxf(len, 0.f), C.W * 0.99999994f);
     if (TRACK) {
-        if (b0 < 0 && b0 + m >= 0) c.below[j] = k - k_begin + 1;
-        if (b0 < C.n_bins && b0 + m >= C.n_bins) c.above[j] = k_end - k + 1;
+        if (b0 < 0 && b0 + m >= 0) cold.set(j, kBelow, k - k_begin + 1);
+        if (b0 < C.n_bins && b0 + m >= C.n_bins) cold.set(j, kAbove, k_end - k + 1);
     }
 }
 
@@ -320,9 +338,9 @@ enum { kFast = 0, kExact = 1 };
 // flushes the bin and starts the next one with the rest of the interval.  LAST: the interval ends
 // on the exact FP64 anchors.  TRACK: bins may lie outside the window (checked, clipped intervals
 // counted).  ok: kExact only, false from the interval that stopped the fast walk onwards.
-template <int NC, int MODE, bool LAST, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& C, const int* bo_end,
-                                     const float* f_end, int k, int k_begin, int k_end, bool* ok, float ramp)
+template <int NC, int NT, int MODE, bool LAST, bool TRACK, bool FF, int LIN>
+__device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& C, const Cold<NC, NT>& cold, int k,
+                                     int k_begin, int k_end, bool* ok, float ramp)
 {
     constexpr int NF = FF ? 3 : 6;                  // carried field components (far field: E only)
     constexpr bool QUAD = LIN == 2;                 // quadratic interpolation (RD_QUADRATIC)
@@ -340,7 +358,7 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
             field_at(r, c.px[j], c.py[j], c.pz[j], c.rpd[j], C, o[j]);
         float t;
         if (LAST) {
-            t = fmaf((float)(bo_end[j] - c.bo[j]), C.W, f_end[j]);
+            t = fmaf((float)(cold.bo_end(j) - c.bo[j]), C.W, cold.f_end(j));
             if (MODE == kFast) t = c.f[j] == -INFINITY ? -INFINITY : t;
         } else {
             t = fmaf(o[j].num, o[j].rden, c.f[j]);
@@ -387,9 +405,10 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
             if (LIN)
-                multi_edges_lin<NC, TRACK, FF, QUAD>(c, j, G[j], D2[j], L[j], inv2L[j], C, fn[j], k, k_begin, k_end);
+                multi_edges_lin<NC, NT, TRACK, FF, QUAD>(c, cold, j, G[j], D2[j], L[j], inv2L[j], C, fn[j], k, k_begin,
+                                                         k_end);
             else
-                multi_edges<NC, TRACK, FF>(c, j, o[j], C, fn[j], k, k_begin, k_end);
+                multi_edges<NC, NT, TRACK, FF>(c, cold, j, o[j], C, fn[j], k, k_begin, k_end);
         }
     }
 #pragma unroll
@@ -403,7 +422,7 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
                 const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
                 float bb[3];
                 bin_b<NC, FF>(c, j, e, cb, bb);
-                if (bin_ok(C, c.bo[j] - c.rb[j])) {
+                if (!RD_CHECK || bin_ok(C, c.bo[j] - row_base<NT>(j, C.n_bins))) {
                     red_add_v4(a, e[0], e[1], e[2], bb[0]);
                     red_add_v2(a + 4, bb[1], bb[2]);
                 }
@@ -432,7 +451,7 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
                 c.f[j] = fn[j];
             }
         } else {
-            const int b = c.bo[j] - c.rb[j];
+            const int b = TRACK || RD_CHECK ? c.bo[j] - row_base<NT>(j, C.n_bins) : 0;
             const bool go = MODE == kFast || !ok[j];
             const bool pr = cr && go && (TRACK ? (unsigned)b < (unsigned)C.n_bins : (!RD_CHECK || bin_ok(C, b)));
             float* a = bin_addr(C, c.bo[j]);
@@ -463,8 +482,8 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
             }
             c.f[j] = cr ? rem : fn[j];
             if (TRACK) {
-                if (cr && b == -1) c.below[j] = k - k_begin + 1;
-                if (cr && b == C.n_bins - 1) c.above[j] = k_end - k + 1;
+                if (cr && b == -1) cold.set(j, kBelow, k - k_begin + 1);
+                if (cr && b == C.n_bins - 1) cold.set(j, kAbove, k_end - k + 1);
             }
             c.bo[j] += cr ? 1 : 0;
         }
@@ -484,12 +503,234 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
 #endif
 constexpr int kUnroll = RD_UNROLL > 0 ? RD_UNROLL : 1;   // samples per loop iteration
 
+// ---------------------------------------------------------------------------------------------
+// Two cells per thread as packed pairs, two intervals at a time (the unchecked walk of the held field).
+//
+// What bounds the walk is the register file: a three-operand FP32 instruction whose operands are all
+// different registers takes 1.7 issue cycles on this part (1.2 with two operands reused; measured with
+// independent chains), so the scalar step's 74 instructions per 32 (cell, interval) pairs read about
+// 165 registers and ran at 93 cycles, 0.8 of the issue slots.  Two-wide instructions (fma.rn.f32x2 and
+// its kin, rounded like the scalar ones) read a sample's constant once for both cells, and two intervals
+// per crossing update halve its reductions, branches and addressing: 50 instructions and 86 cycles.
+// Measured on 1000 electrons x 4000 steps x 16384 cells x 2048 bins: 149.9 -> 139.0 ms per launch; two
+// cells packed, one interval at a time: 154.4 ms; accumulators packed as well: 141.7 ms (their halves
+// are written one by one on a crossing, which costs a copy of every accumulator per pass); one crossing
+// update for both cells with selects: 155 ms.  128 registers (4 CTAs of 128 threads per SM) rather than
+// 96 (5 CTAs: 143.4 ms with packed accumulators).
+// ---------------------------------------------------------------------------------------------
+__device__ __forceinline__ float2 fma2(float2 a, float2 b, float2 c)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 A, B, C, D;\n\tmov.b64 A, {%2, %3};\n\tmov.b64 B, {%4, %5};\n\tmov.b64 C, {%6, %7};\n\t"
+        "fma.rn.ftz.f32x2 D, A, B, C;\n\tmov.b64 {%0, %1}, D;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y), "f"(c.x), "f"(c.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 mul2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 A, B, D;\n\tmov.b64 A, {%2, %3};\n\tmov.b64 B, {%4, %5};\n\t"
+        "mul.rn.ftz.f32x2 D, A, B;\n\tmov.b64 {%0, %1}, D;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 add2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 A, B, D;\n\tmov.b64 A, {%2, %3};\n\tmov.b64 B, {%4, %5};\n\t"
+        "add.rn.ftz.f32x2 D, A, B;\n\tmov.b64 {%0, %1}, D;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+
+__device__ __forceinline__ float2 both(float v) { return make_float2(v, v); }
+__device__ __forceinline__ float2 sub2(float2 a, float2 b)
+{
+    float2 d;
+    asm("{\n\t.reg .b64 A, B, D;\n\tmov.b64 A, {%2, %3};\n\tmov.b64 B, {%4, %5};\n\t"
+        "sub.rn.ftz.f32x2 D, A, B;\n\tmov.b64 {%0, %1}, D;\n\t}"
+        : "=f"(d.x), "=f"(d.y)
+        : "f"(a.x), "f"(a.y), "f"(b.x), "f"(b.y));
+    return d;
+}
+__device__ __forceinline__ float2 rcp2(float2 a) { return make_float2(fast_rcp(a.x), fast_rcp(a.y)); }
+__device__ __forceinline__ float2 pair_of(const float (&v)[2]) { return make_float2(v[0], v[1]); }
+__device__ __forceinline__ void set_pair(float (&v)[2], float2 a)
+{
+    v[0] = a.x;
+    v[1] = a.y;
+}
+
+struct Field2 {
+    float2 E[3], B[3], S, rinv, num, rden;      // as Field, for both cells (far-field limit: B, rinv unused)
+};
+
+// field_at / field_at_ff for the two cells, with the same operations in the same order.
+template <bool FF>
+__device__ __forceinline__ void field_pair(const RecS& r, Cells<2>& c, const Consts& C, Field2& o)
+{
+    if (FF) {
+        const float2 nx = pair_of(c.px), ny = pair_of(c.py), nz = pair_of(c.pz);
+        const float2 bx = add2(add2(nx, both(r.nbx)), pair_of(c.nlx)), by = add2(add2(ny, both(r.nby)), pair_of(c.nly)),
+                     bz = add2(add2(nz, both(r.nbz)), pair_of(c.nlz));
+        const float2 nb2 = fma2(bx, bx, fma2(by, by, mul2(bz, bz)));
+        o.num = fma2(bx, both(r.d2x), fma2(by, both(r.d2y), fma2(bz, both(r.d2z), add2(nb2, both(r.gd)))));
+        o.rden = both(0.5f);
+        const float2 ikn = rcp2(fma2(nb2, both(-0.5f), both(r.nhig2)));
+        o.S = mul2(mul2(ikn, ikn), pair_of(c.rpd));
+        const float2 c1n = mul2(fma2(nx, both(r.bdx), fma2(ny, both(r.bdy), mul2(nz, both(r.bdz)))), ikn);
+        o.E[0] = fma2(bx, c1n, both(r.bdx));
+        o.E[1] = fma2(by, c1n, both(r.bdy));
+        o.E[2] = fma2(bz, c1n, both(r.bdz));
+        return;
+    }
+    const float2 dx = add2(pair_of(c.px), both(r.nx)), dy = add2(pair_of(c.py), both(r.ny)),
+                 dz = add2(pair_of(c.pz), both(r.nz));
+    const float2 r2 = fma2(dx, dx, fma2(dy, dy, mul2(dz, dz)));
+    const float2 rinv = make_float2(fast_rsqrt(r2.x), fast_rsqrt(r2.y));
+    const float2 bx = fma2(dx, rinv, both(r.nbx)), by = fma2(dy, rinv, both(r.nby)), bz = fma2(dz, rinv, both(r.nbz));
+    const float2 nb2 = fma2(bx, bx, fma2(by, by, mul2(bz, bz)));
+    const float2 gg = fma2(bx, both(r.d2x), fma2(by, both(r.d2y), fma2(bz, both(r.d2z), add2(nb2, both(r.gd)))));
+    o.num = fma2(both(r.dtg), rinv, gg);
+    o.rden = rcp2(fma2(pair_of(c.rpd), rinv, both(1.f)));
+    set_pair(c.rpd, fma2(r2, rinv, both(C.DT)));
+    const float2 kn = fma2(nb2, both(-0.5f), both(r.nhig2));
+    const float2 ikn = rcp2(kn);
+    const float2 nrik = mul2(rinv, ikn);
+    o.S = mul2(nrik, ikn);
+    const float2 c1n = mul2(fma2(dx, both(r.bdx), fma2(dy, both(r.bdy), fma2(dz, both(r.bdz), both(r.ig2n)))), nrik);
+    o.E[0] = fma2(bx, c1n, both(r.bdx));
+    o.E[1] = fma2(by, c1n, both(r.bdy));
+    o.E[2] = fma2(bz, c1n, both(r.bdz));
+    // d x E'; the negated products are written as 0 - product, which the subtraction absorbs (a sign
+    // flip of each half would be two more instructions)
+    const float2 zero = both(0.f);
+    o.B[0] = fma2(dy, o.E[2], sub2(zero, mul2(dz, o.E[1])));
+    o.B[1] = fma2(dz, o.E[0], sub2(zero, mul2(dx, o.E[2])));
+    o.B[2] = fma2(dx, o.E[1], sub2(zero, mul2(dy, o.E[0])));
+    o.rinv = rinv;
+}
+
+// acc += weight (per unit S) times the field, both cells.
+template <bool FF>
+__device__ __forceinline__ void add_field(Cells<2>& c, const Field2& o, float2 w)
+{
+    const float2 ws = mul2(w, o.S), wb = FF ? ws : mul2(ws, o.rinv);
+#pragma unroll
+    for (int i = 0; i < 3; ++i) {
+        c.acc[i][0] = fmaf(o.E[i].x, ws.x, c.acc[i][0]);
+        c.acc[i][1] = fmaf(o.E[i].y, ws.y, c.acc[i][1]);
+        if (!FF) {
+            c.acc[3 + i][0] = fmaf(o.B[i].x, wb.x, c.acc[3 + i][0]);
+            c.acc[3 + i][1] = fmaf(o.B[i].y, wb.y, c.acc[3 + i][1]);
+        }
+    }
+}
+
+__device__ __forceinline__ float half_of(float2 a, int j) { return j == 0 ? a.x : a.y; }
+
+// Add the bin cell j is filling to global memory (the bin is inside the window).
+template <int NT, bool FF>
+__device__ __forceinline__ void red_bin(const Consts& C, const Cells<2>& c, int j)
+{
+    if (RD_CHECK && !bin_ok(C, c.bo[j] - row_base<NT>(j, C.n_bins))) return;
+    float* a = bin_addr(C, c.bo[j]);
+    const float e[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
+    const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
+    float b[3];
+    bin_b<2, FF>(c, j, e, cb, b);
+    red_add_v4(a, e[0], e[1], e[2], b[0]);
+    red_add_v2(a + 4, b[1], b[2]);
+}
+
+// The deposit of one interval (the fast, unchecked step) from the fields of its sample.
+template <int NT, bool FF>
+__device__ __forceinline__ void deposit_pair(Cells<2>& c, const Field2& o, const Consts& C)
+{
+    const float2 t = fma2(o.num, o.rden, pair_of(c.f));
+    add_field<FF>(c, o, sub2(make_float2(fminf(t.x, C.W), fminf(t.y, C.W)), pair_of(c.f)));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        float fn = half_of(t, j);
+        fn = fn < 2.f * C.W ? fn : -INFINITY;
+        c.f[j] = fn;
+        if (fn >= C.W) {
+            red_bin<NT, FF>(C, c, j);
+            const float rem = fn - C.W;
+            const float rs = rem * half_of(o.S, j), rbw = FF ? rs : rs * half_of(o.rinv, j);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                c.acc[i][j] = half_of(o.E[i], j) * rs;
+                if (!FF) c.acc[3 + i][j] = half_of(o.B[i], j) * rbw;
+            }
+            c.f[j] = rem;
+            c.bo[j] += 1;
+        }
+    }
+}
+
+// Two intervals (samples ra, then rb) at once.  A cell whose two intervals pass at most one bin edge
+// needs one crossing update for both: the bin being filled takes the parts of both intervals below the
+// edge, is flushed, and the next bin starts with the parts above it.  The arrival times and bins equal
+// those of two single steps bit for bit (the exact re-walk of a tile relies on it).  A warp with a cell
+// that passes two edges takes the two single steps instead.
+template <int NT, bool FF>
+__device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, const RecS& rb, const Consts& C)
+{
+    Field2 a, b;
+    field_pair<FF>(ra, c, C, a);
+    field_pair<FF>(rb, c, C, b);
+    const float2 t1 = fma2(a.num, a.rden, pair_of(c.f));
+    const bool c1x = t1.x >= C.W, c1y = t1.y >= C.W;            // the first interval passes the edge
+    const float2 r1 = add2(t1, both(-C.W));
+    const float2 f1 = make_float2(c1x ? r1.x : t1.x, c1y ? r1.y : t1.y);
+    const float2 t2 = fma2(b.num, b.rden, f1);
+    // false for a NaN too (the single steps stop such a cell)
+    const bool ok = t2.x < (c1x ? C.W : 2.f * C.W) && t2.y < (c1y ? C.W : 2.f * C.W);
+    if (!__all_sync(0xffffffffu, ok)) {
+        deposit_pair<NT, FF>(c, a, C);
+        deposit_pair<NT, FF>(c, b, C);
+        return;
+    }
+    const float2 m1 = make_float2(fminf(t1.x, C.W), fminf(t1.y, C.W));
+    const float2 m2 = make_float2(fminf(t2.x, C.W), fminf(t2.y, C.W));
+    const float2 wf = sub2(m2, f1);
+    add_field<FF>(c, a, sub2(m1, pair_of(c.f)));
+    add_field<FF>(c, b, make_float2(c1x ? 0.f : wf.x, c1y ? 0.f : wf.y));
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const bool c1 = j == 0 ? c1x : c1y;
+        const float tt = half_of(t2, j);
+        c.f[j] = tt;
+        if (c1 || tt >= C.W) {
+            red_bin<NT, FF>(C, c, j);
+            const float r2 = tt - C.W;
+            const float wa = c1 ? half_of(r1, j) : 0.f;
+            const float wb = c1 ? half_of(wf, j) : r2;
+            const float sa = wa * half_of(a.S, j), sb = wb * half_of(b.S, j);
+            const float ba = FF ? sa : sa * half_of(a.rinv, j), bb = FF ? sb : sb * half_of(b.rinv, j);
+#pragma unroll
+            for (int i = 0; i < 3; ++i) {
+                c.acc[i][j] = fmaf(half_of(b.E[i], j), sb, half_of(a.E[i], j) * sa);
+                if (!FF) c.acc[3 + i][j] = fmaf(half_of(b.B[i], j), bb, half_of(a.B[i], j) * ba);
+            }
+            c.f[j] = c1 ? tt : r2;
+            c.bo[j] += 1;
+        }
+    }
+}
+
 // Per-thread copy of the walk state at the start of a tile, in shared memory ([word][thread]):
 // f, rpd, bo, below, above, acc[6], gp[6], and for the quadratic interpolation gpp[6], hp.
 constexpr int save_cell(int lin) { return lin == 2 ? 24 : 17; }
 
-template <int NC, int NT, bool FF, int LIN>
-__device__ __forceinline__ void save_state(const Cells<NC>& c, float (*sv)[NT], int tid)
+template <int NC, int NT, bool TRACK, bool FF, int LIN>
+__device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT>& cold, float (*sv)[NT], int tid)
 {
     constexpr int NF = FF ? 3 : 6;
     constexpr int kSaveCell = save_cell(LIN);
@@ -498,8 +739,10 @@ __device__ __forceinline__ void save_state(const Cells<NC>& c, float (*sv)[NT], 
         sv[j * kSaveCell + 0][tid] = c.f[j];
         sv[j * kSaveCell + 1][tid] = c.rpd[j];
         sv[j * kSaveCell + 2][tid] = __int_as_float(c.bo[j]);
-        sv[j * kSaveCell + 3][tid] = __int_as_float(c.below[j]);
-        sv[j * kSaveCell + 4][tid] = __int_as_float(c.above[j]);
+        if (TRACK) {
+            sv[j * kSaveCell + 3][tid] = __int_as_float(cold.below(j));
+            sv[j * kSaveCell + 4][tid] = __int_as_float(cold.above(j));
+        }
 #pragma unroll
         for (int i = 0; i < NF; ++i) sv[j * kSaveCell + 5 + i][tid] = c.acc[i][j];
         if (LIN) {
@@ -514,8 +757,8 @@ __device__ __forceinline__ void save_state(const Cells<NC>& c, float (*sv)[NT], 
     }
 }
 
-template <int NC, int NT, bool FF, int LIN>
-__device__ __forceinline__ void restore_state(Cells<NC>& c, float (*sv)[NT], int tid)
+template <int NC, int NT, bool TRACK, bool FF, int LIN>
+__device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& cold, float (*sv)[NT], int tid)
 {
     constexpr int NF = FF ? 3 : 6;
     constexpr int kSaveCell = save_cell(LIN);
@@ -524,8 +767,10 @@ __device__ __forceinline__ void restore_state(Cells<NC>& c, float (*sv)[NT], int
         c.f[j] = sv[j * kSaveCell + 0][tid];
         c.rpd[j] = sv[j * kSaveCell + 1][tid];
         c.bo[j] = __float_as_int(sv[j * kSaveCell + 2][tid]);
-        c.below[j] = __float_as_int(sv[j * kSaveCell + 3][tid]);
-        c.above[j] = __float_as_int(sv[j * kSaveCell + 4][tid]);
+        if (TRACK) {
+            cold.set(j, kBelow, sv[j * kSaveCell + 3][tid]);
+            cold.set(j, kAbove, sv[j * kSaveCell + 4][tid]);
+        }
 #pragma unroll
         for (int i = 0; i < NF; ++i) c.acc[i][j] = sv[j * kSaveCell + 5 + i][tid];
         if (LIN) {
@@ -542,31 +787,39 @@ __device__ __forceinline__ void restore_state(Cells<NC>& c, float (*sv)[NT], int
 
 template <int NC, int NT, bool TRACK, bool FF, int LIN>
 __device__ __forceinline__ void walk_tile(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
-                                          float ramp, const int* bo_end, const float* f_end, int k0, int k_begin,
-                                          int k_end, float (*sv)[NT])
+                                          float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
+                                          float (*sv)[NT])
 {
     const int tid = threadIdx.x;
     const int n_regular = last_tile ? cnt - 1 : cnt;
-    save_state<NC, NT, FF, LIN>(c, sv, tid);
+    save_state<NC, NT, TRACK, FF, LIN>(c, cold, sv, tid);
     bool ok[NC];
+    if constexpr (NC == 2 && !TRACK && LIN == 0) {
+        int i = 0;
+#pragma unroll 1
+        for (; i + 1 < n_regular; i += 2) two_steps_pair<NT, FF>(c, tile[i], tile[i + 1], C);
+        if (i < n_regular)
+            step<NC, NT, kFast, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
+    } else {
 #pragma unroll kUnroll
-    for (int i = 0; i < n_regular; ++i)
-        step<NC, kFast, false, TRACK, FF, LIN>(c, tile[i], C, bo_end, f_end, k0 + i, k_begin, k_end, ok, ramp);
+        for (int i = 0; i < n_regular; ++i)
+            step<NC, NT, kFast, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
+    }
     if (last_tile)
-        step<NC, kFast, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, bo_end, f_end, k_end, k_begin, k_end, ok, ramp);
+        step<NC, NT, kFast, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp);
     bool stopped = false;
 #pragma unroll
     for (int j = 0; j < NC; ++j) stopped = stopped || c.f[j] == -INFINITY;
     if (__any_sync(0xffffffffu, stopped)) {
         // some interval of a cell of this warp passed two or more bin edges: walk the tile again
-        restore_state<NC, NT, FF, LIN>(c, sv, tid);
+        restore_state<NC, NT, TRACK, FF, LIN>(c, cold, sv, tid);
 #pragma unroll
         for (int j = 0; j < NC; ++j) ok[j] = true;
 #pragma unroll 1
         for (int i = 0; i < n_regular; ++i)
-            step<NC, kExact, false, TRACK, FF, LIN>(c, tile[i], C, bo_end, f_end, k0 + i, k_begin, k_end, ok, ramp);
+            step<NC, NT, kExact, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
         if (last_tile)
-            step<NC, kExact, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, bo_end, f_end, k_end, k_begin, k_end, ok, ramp);
+            step<NC, NT, kExact, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp);
     }
 }
 
@@ -616,8 +869,7 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
 
     // anchors: exact FP64 arrival (bins) at both ends of the chunk, per cell
     Cells<NC> c;
-    int bo_end[NC];
-    float f_end[NC];
+    const Cold<NC, NT> cold{sv + NC * save_cell(LIN)};
     float hp0[NC];                              // quadratic: length of interval k_begin - 1 (dt units)
     bool partial = false;
     unsigned long long clip = 0, crossed = 0;
@@ -628,17 +880,15 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         const int cell = cb * CPC + row;
         // a cell without arrivals in the window still walks (no per-cell branch in the step) but
         // from a time that never reaches a bin edge: nothing is flushed
-        c.rb[j] = row * P.n_bins;
-        c.bo[j] = c.rb[j];
-        c.live[j] = false;
-        c.below[j] = c.above[j] = 0;
+        const int rb = row * P.n_bins;
+        c.bo[j] = rb;
         c.f[j] = -1e30f;
         c.rpd[j] = 1e6f;
         c.px[j] = 1e6f;
         c.py[j] = c.pz[j] = 0.f;
         c.nlx[j] = c.nly[j] = c.nlz[j] = 0.f;
-        bo_end[j] = c.bo[j];
-        f_end[j] = 0.f;
+        int bo_end = rb, below = -1;
+        float f_end = 0.f;
 #pragma unroll
         for (int i = 0; i < 6; ++i) c.acc[i][j] = 0.f;
         if (cell < P.n_pix) {
@@ -654,9 +904,9 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
                 ua = arrival_bins(xa[0], xa[1], xa[2], cl, P.t0, k_begin - 1, P.dt, P.inv_dt_det, Ra);
                 ue = arrival_bins(xe[0], xe[1], xe[2], cl, P.t0, k_end, P.dt, P.inv_dt_det, Re);
             }
-            c.live[j] = (ue > 0.0) && (ua < (double)P.n_bins);
+            const bool live = (ue > 0.0) && (ua < (double)P.n_bins);
             hp0[j] = 1.f;
-            if (q_prev && c.live[j]) {
+            if (q_prev && live) {
                 const double* xq = xp + 3 * (size_t)(k_begin - 2);
                 double Rq;
                 const double uq =
@@ -665,14 +915,14 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
                        : arrival_bins(xq[0], xq[1], xq[2], cl, P.t0, k_begin - 2, P.dt, P.inv_dt_det, Rq);
                 hp0[j] = (float)((ua - uq) * P.W);
             }
-            if (!c.live[j]) {
+            if (!live) {
                 clip += (unsigned long long)n_int;
             } else {
                 const double fla = floor(ua), fle = floor(ue);
-                c.bo[j] = c.rb[j] + walk_bin(fla);
+                c.bo[j] = rb + walk_bin(fla);
                 c.f[j] = (float)(ua - fla) * P.W;
-                bo_end[j] = c.rb[j] + walk_bin(fle);
-                f_end[j] = (float)(ue - fle) * P.W;
+                bo_end = rb + walk_bin(fle);
+                f_end = (float)(ue - fle) * P.W;
                 if (FF) {
                     c.px[j] = (float)ncx;
                     c.py[j] = (float)ncy;
@@ -687,14 +937,23 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
                     c.py[j] = (float)cl.y;
                     c.pz[j] = (float)cl.z;
                 }
-                c.below[j] = (ua < 0.0) ? n_int : 0;
+                below = (ua < 0.0) ? n_int : 0;
                 // unchecked bins need a margin of one bin to each window edge (the FP32 walk may
                 // drift by far less than a bin before the end anchor corrects it)
                 partial = partial || (ua < 1.0) || (ue > (double)P.n_bins - 1.0);
-                crossed += (unsigned long long)max(0, bo_end[j] - c.bo[j]);
+                crossed += (unsigned long long)max(0, bo_end - c.bo[j]);
             }
         }
+        cold.set(j, kBoEnd, bo_end);
+        cold.set(j, kFEnd, f_end);
+        cold.set(j, kBelow, below);
+        cold.set(j, kAbove, 0);
     }
+    if (clip) atomicAdd(&P.counters->clipped, clip);
+    // warp-aggregated count of bin edges crossed (bins touched = intervals + crossings)
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) crossed += __shfl_xor_sync(0xffffffffu, crossed, o);
+    if ((tid & 31) == 0 && crossed) atomicAdd(&P.counters->crossings, crossed);
     // clip tracking costs instructions in the bin-crossing path: only CTAs that need it use it
     if (LIN) {
         // field of the sample before the chunk; a trajectory's first interval holds F_1 (sample 0
@@ -750,11 +1009,11 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         const int cnt = min(kTileSteps, k_end - k0 + 1);
         const bool last_tile = (t == n_tiles - 1);
         if (track)
-            walk_tile<NC, NT, true, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, bo_end, f_end, k0,
-                                     k_begin, k_end, sv);
+            walk_tile<NC, NT, true, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, cold, k0,
+                                          k_begin, k_end, sv);
         else
-            walk_tile<NC, NT, false, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, bo_end, f_end, k0,
-                                      k_begin, k_end, sv);
+            walk_tile<NC, NT, false, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, cold, k0,
+                                          k_begin, k_end, sv);
         __syncthreads();
         if (tid == 0 && t + 2 < n_tiles) {
             fence_proxy_async();
@@ -765,19 +1024,17 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         }
     }
     g_base += (unsigned)n_tiles;
-    // close the last bin; count clipped intervals and crossed bin edges
+    // close the last bin; count clipped intervals
+    unsigned long long clipped = 0;
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
-        if (c.live[j]) {
-            flush_acc<NC, FF>(C, c, j, c.bo[j] - c.rb[j], c.bo[j]);
-            clip += (unsigned long long)min(n_int, c.below[j] + c.above[j]);
+        const int below = cold.below(j);
+        if (below >= 0) {
+            flush_acc<NC, FF>(C, c, j, c.bo[j] - row_base<NT>(j, P.n_bins), c.bo[j]);
+            clipped += (unsigned long long)min(n_int, below + cold.above(j));
         }
     }
-    if (clip) atomicAdd(&P.counters->clipped, clip);
-    // warp-aggregated count of bin edges crossed (bins touched = intervals + crossings)
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) crossed += __shfl_xor_sync(0xffffffffu, crossed, o);
-    if ((tid & 31) == 0 && crossed) atomicAdd(&P.counters->crossings, crossed);
+    if (clipped) atomicAdd(&P.counters->clipped, clipped);
     return true;
 }
 
@@ -791,23 +1048,31 @@ __device__ __forceinline__ void init_staging(uint64_t* bar)
     __syncthreads();
 }
 
-// Resident CTAs per SM the register allotment must allow: about 640 threads, as for the default
-// shape (2 cells per thread, 256 cells per CTA: 128 threads, 5 CTAs).
+// Resident CTAs per SM the register allotment must allow.  The default CTA (128 threads): 4 for the held
+// field's paired walk and the quadratic walk (their state needs 110-128 registers), else 5; other CTA
+// sizes: about 640 threads per SM.
 #ifndef RD_QUAD_MINBLOCKS
-#define RD_QUAD_MINBLOCKS 4      // the quadratic walk's CTAs per SM (its state needs more than 96 registers)
+#define RD_QUAD_MINBLOCKS 4
 #endif
-constexpr int mixed_min_blocks(int nt, int lin = 0)
+#ifndef RD_FF_MINBLOCKS
+#define RD_FF_MINBLOCKS 5
+#endif
+#ifndef RD_LIN_MINBLOCKS
+#define RD_LIN_MINBLOCKS 4
+#endif
+constexpr int mixed_min_blocks(int nt, bool ff, int lin)
 {
-    return nt >= 128 ? (nt == 128 ? (lin == 2 ? RD_QUAD_MINBLOCKS : RD_MIXED_MINBLOCKS) : 640 / nt) : 640 / nt;
+    if (nt != 128) return 640 / nt;
+    return lin == 2 ? RD_QUAD_MINBLOCKS : lin == 1 ? RD_LIN_MINBLOCKS : ff ? RD_FF_MINBLOCKS : RD_MIXED_MINBLOCKS;
 }
 
 template <bool FF, int LIN, int NC, int CPC>
-__global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, LIN)) k_deposit_mixed(const DepositParams P)
+__global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, FF, LIN)) k_deposit_mixed(const DepositParams P)
 {
     constexpr int NT = CPC / NC;
     __shared__ __align__(128) RecS tile[2][kTileSteps];
     __shared__ __align__(8) uint64_t bar[2];
-    __shared__ float sv[NC * save_cell(LIN)][NT];
+    __shared__ float sv[NC * (save_cell(LIN) + kColdWords)][NT];
     init_staging(bar);
     int p, cb, ch;
     item_coords(blockIdx.x, P, p, cb, ch);
@@ -823,14 +1088,14 @@ __global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, LIN)) k_d
 // state.  (Drawing the next item while walking the current one measured 8 % slower: the drawing
 // thread then waits on the atomic before it issues the current item's record copies.)
 template <bool FF, int LIN>
-__global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads, LIN))
+__global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads, FF, LIN))
     k_deposit_batch(const DepositParams* __restrict__ probs, const long long* __restrict__ item_off, int n_probs,
                     unsigned long long* next_item)
 {
     __shared__ __align__(128) RecS tile[2][kTileSteps];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ long long s_next;
-    __shared__ float sv[kMixedCells * save_cell(LIN)][kMixedThreads];
+    __shared__ float sv[kMixedCells * (save_cell(LIN) + kColdWords)][kMixedThreads];
     init_staging(bar);
     const long long total = item_off[n_probs];
     unsigned g = 0;
