@@ -162,50 +162,60 @@ struct __align__(16) RecC {
 };
 static_assert(sizeof(RecC) == 128, "RecC must be 128 bytes");
 
-__global__ void k_precompute_comp(const double* __restrict__ x, const double* __restrict__ u, int n_part,
+// One sample per lane, the previous sample's beta from the lane below (lane 0 only provides one): see
+// k_precompute_mixed.
+__global__ void k_precompute_comp(const double* __restrict__ x, const double* __restrict__ u, long long total,
                                   int n_samples, double dt, int flags, RecC* __restrict__ rec, DevCounters* counters)
 {
-    const long long total = (long long)n_part * n_samples;
     const bool far_on = (flags & RD_FAR) != 0;
     const double inv_dt = 1.0 / dt;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(i % n_samples);
-        const double* xk = x + 3 * i;
-        const double* uk = u + 3 * i;
-        bool bad = !(isfinite(xk[0]) && isfinite(xk[1]) && isfinite(xk[2]) && isfinite(uk[0]) && isfinite(uk[1]) &&
-                     isfinite(uk[2]));
-        const double uu = uk[0] * uk[0] + uk[1] * uk[1] + uk[2] * uk[2];
-        const double gam = sqrt(1.0 + uu);
-        const double b[3] = {uk[0] / gam, uk[1] / gam, uk[2] / gam};
-        double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, g = 1.0;
-        if (k > 0) {
-            const double* up = uk - 3;
-            const double gp = sqrt(1.0 + (up[0] * up[0] + up[1] * up[1] + up[2] * up[2]));
-            for (int c = 0; c < 3; ++c) {
-                a[c] = (b[c] - up[c] / gp) * inv_dt;
-                v[c] = (xk[c] - xk[c - 3]) * inv_dt;
-            }
-            g = 1.0 - (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
-            bad = bad || !(g > 0.0);
-        }
-        if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
-        RecC r;
-        double e2 = 0.0;
+    const int lane = threadIdx.x & 31;
+    const long long i = ((blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5) * kPrecomputeSpan - 1 + lane;
+    const bool in = i >= 0 && i < total;
+    double xk[3] = {0.0, 0.0, 0.0}, uk[3] = {0.0, 0.0, 0.0};
+    if (in) {
         for (int c = 0; c < 3; ++c) {
-            const double e = b[c] - v[c];
-            e2 += e * e;
-            r.x[c] = df_from_double(xk[c]);
-            r.b[c] = df_from_double(b[c]);
-            r.bd[c] = df_from_double(far_on ? a[c] : 0.0);
-            r.d2[c] = df_from_double(2.0 * e);
+            xk[c] = x[3 * i + c];
+            uk[c] = u[3 * i + c];
         }
-        r.ig2 = df_from_double(1.0 / (1.0 + uu));
-        r.ig = df_from_double(1.0 / gam);
-        r.dtg = df_from_double(dt * g);
-        r.gd = df_from_double(g + e2);
-        rec[i] = r;
     }
+    const double uu = uk[0] * uk[0] + uk[1] * uk[1] + uk[2] * uk[2];
+    const double gam = sqrt(1.0 + uu);
+    const double b[3] = {uk[0] / gam, uk[1] / gam, uk[2] / gam};
+    double bp[3], xp[3];
+    for (int c = 0; c < 3; ++c) {
+        bp[c] = __shfl_up_sync(0xffffffffu, b[c], 1);
+        xp[c] = __shfl_up_sync(0xffffffffu, xk[c], 1);
+    }
+    if (!in || lane == 0) return;
+    const int k = (int)(i % n_samples);
+    bool bad = !(isfinite(xk[0]) && isfinite(xk[1]) && isfinite(xk[2]) && isfinite(uk[0]) && isfinite(uk[1]) &&
+                 isfinite(uk[2]));
+    double a[3] = {0.0, 0.0, 0.0}, v[3] = {0.0, 0.0, 0.0}, g = 1.0;
+    if (k > 0) {
+        for (int c = 0; c < 3; ++c) {
+            a[c] = (b[c] - bp[c]) * inv_dt;
+            v[c] = (xk[c] - xp[c]) * inv_dt;
+        }
+        g = 1.0 - (v[0] * v[0] + v[1] * v[1] + v[2] * v[2]);
+        bad = bad || !(g > 0.0);
+    }
+    if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
+    RecC r;
+    double e2 = 0.0;
+    for (int c = 0; c < 3; ++c) {
+        const double e = b[c] - v[c];
+        e2 += e * e;
+        r.x[c] = df_from_double(xk[c]);
+        r.b[c] = df_from_double(b[c]);
+        r.bd[c] = df_from_double(far_on ? a[c] : 0.0);
+        r.d2[c] = df_from_double(2.0 * e);
+    }
+    r.ig2 = df_from_double(1.0 / (1.0 + uu));
+    r.ig = df_from_double(1.0 / gam);
+    r.dtg = df_from_double(dt * g);
+    r.gd = df_from_double(g + e2);
+    rec[i] = r;
 }
 
 namespace {
@@ -582,8 +592,8 @@ cudaError_t launch_precompute_comp(const double* x, const double* u, int n_part,
                                    void* rec, DevCounters* counters, cudaStream_t s)
 {
     const long long n = (long long)n_part * n_samples;
-    k_precompute_comp<<<grid_stride_blocks(n, 256, 16), 256, 0, s>>>(x, u, n_part, n_samples, dt, flags,
-                                                                     static_cast<RecC*>(rec), counters);
+    const PrecomputeGrid g(n);
+    k_precompute_comp<<<g.blocks, g.threads, 0, s>>>(x, u, n, n_samples, dt, flags, static_cast<RecC*>(rec), counters);
     return cudaGetLastError();
 }
 

@@ -31,99 +31,151 @@ __device__ __forceinline__ void beta_of(const double* u, double& bx, double& by,
     ig2 = 1.0 / (1.0 + uu);
 }
 
-__device__ __forceinline__ bool finite3(const double* v)
+// The precompute kernels take one sample per lane; a warp covers 31 samples and its lane 0 the one
+// before them, so that the previous sample's beta comes from the neighbouring lane by a shuffle instead
+// of a second evaluation (square root and divisions in FP64, the pipe that bounds these kernels: 4e6
+// samples took 1274 us, five times the time of their bytes).  Returns the flat sample index (particle *
+// n_samples + k) of the lane, -1 beyond the ends; `out` says whether the lane owns the sample.
+__device__ __forceinline__ long long warp_sample(long long total, bool& out)
 {
-    return isfinite(v[0]) && isfinite(v[1]) && isfinite(v[2]);
+    const long long w = (blockIdx.x * (long long)blockDim.x + threadIdx.x) >> 5;
+    const int lane = threadIdx.x & 31;
+    const long long i = w * kPrecomputeSpan - 1 + lane;
+    out = lane > 0 && i < total;
+    return i < total ? i : -1;
 }
 
+// particle and sample of a flat index (32-bit division where it fits: the 64-bit one is ten times longer)
+__device__ __forceinline__ void split_sample(long long i, int n_samples, long long& p, int& k)
+{
+    if (i <= 0xffffffffLL) {
+        const unsigned q = (unsigned)i / (unsigned)n_samples;
+        p = q;
+        k = (int)((unsigned)i - q * (unsigned)n_samples);
+    } else {
+        p = i / n_samples;
+        k = (int)(i - p * n_samples);
+    }
+}
+
+// not finite (infinity or NaN), tested on the exponent bits (integer pipe)
+__device__ __forceinline__ bool not_finite(double v) { return (__double2hiint(v) & 0x7ff00000) == 0x7ff00000; }
+
+__device__ __forceinline__ bool bad3(const double* v) { return not_finite(v[0]) || not_finite(v[1]) || not_finite(v[2]); }
+
 __global__ void k_precompute_mixed(const double* __restrict__ x, const double* __restrict__ u,
-                                   const double* __restrict__ q, double qscale, int n_part, int n_samples,
+                                   const double* __restrict__ q, double qscale, long long total, int n_samples,
                                    double dt, int flags, RecS* __restrict__ rec, DevCounters* counters)
 {
-    const long long total = (long long)n_part * n_samples;
-    const double near_on = (flags & RD_NEAR) ? 1.0 : 0.0;
-    const bool far_on = (flags & RD_FAR) != 0;
+    const bool near_on = (flags & RD_NEAR) != 0, far_on = (flags & RD_FAR) != 0;
     const double inv_dt = 1.0 / dt;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(i % n_samples);
-        // charge factor folded into the betadot and gamma^-2 terms of Eq. 1 (deposit records)
-        const double qf = qscale != 0.0 ? -(q ? q[i / n_samples] : 1.0) * qscale : 1.0;
-        const double* xk = x + 3 * i;
-        const double* uk = u + 3 * i;
-        bool bad = !finite3(xk) || !finite3(uk);
-        double bx, by, bz, ig2;
-        beta_of(uk, bx, by, bz, ig2);
-        double ax = 0.0, ay = 0.0, az = 0.0, vx = 0.0, vy = 0.0, vz = 0.0, g = 1.0;
-        if (k > 0) {
-            double px, py, pz, pig2;
-            beta_of(uk - 3, px, py, pz, pig2);
-            ax = (bx - px) * inv_dt;
-            ay = (by - py) * inv_dt;
-            az = (bz - pz) * inv_dt;
-            vx = (xk[0] - xk[-3]) * inv_dt;
-            vy = (xk[1] - xk[-2]) * inv_dt;
-            vz = (xk[2] - xk[-1]) * inv_dt;
-            g = 1.0 - (vx * vx + vy * vy + vz * vz);
-            bad = bad || !(g > 0.0);
+    bool out;
+    const long long i = warp_sample(total, out);
+    double xk[3] = {0.0, 0.0, 0.0}, uk[3] = {0.0, 0.0, 0.0};
+    if (i >= 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            xk[c] = x[3 * i + c];
+            uk[c] = u[3 * i + c];
         }
-        if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
-        // delta = beta_k - vbar_k (difference of end-point and chord velocities)
-        const double ex = bx - vx, ey = by - vy, ez = bz - vz;
-        auto put = [](double v) { return (float)v; };
-        RecS r;
-        r.nx = put(-xk[0]);
-        r.ny = put(-xk[1]);
-        r.nz = put(-xk[2]);
-        r.nhig2 = put(-0.5 * ig2);
-        r.nbx = put(-bx);
-        r.nby = put(-by);
-        r.nbz = put(-bz);
-        r.ig2n = put(qf * (near_on * ig2));
-        r.bdx = put(far_on ? qf * ax : 0.0);
-        r.bdy = put(far_on ? qf * ay : 0.0);
-        r.bdz = put(far_on ? qf * az : 0.0);
-        r.dtg = put(dt * g);
-        r.d2x = put(2.0 * ex);
-        r.d2y = put(2.0 * ey);
-        r.d2z = put(2.0 * ez);
-        r.gd = put(g + (ex * ex + ey * ey + ez * ez));
-        rec[i] = r;
     }
+    // beta = u / gamma, gamma^-1 = (1 + u^2)^(-1/2): the records are FP32, one ulp of FP64 more or less
+    // in gamma^-1 does not show in them
+    const double rg = rsqrt(fma(uk[0], uk[0], fma(uk[1], uk[1], fma(uk[2], uk[2], 1.0))));
+    const double ig2 = rg * rg;
+    double b[3], db[3], dx[3];
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+        b[c] = uk[c] * rg;
+        db[c] = b[c] - __shfl_up_sync(0xffffffffu, b[c], 1);
+        dx[c] = xk[c] - __shfl_up_sync(0xffffffffu, xk[c], 1);
+    }
+    if (!out) return;
+    long long p;
+    int k;
+    split_sample(i, n_samples, p, k);
+    // charge factor folded into the betadot and gamma^-2 terms of Eq. 1 (deposit records)
+    const double qf = qscale != 0.0 ? -(q ? q[p] : 1.0) * qscale : 1.0;
+    bool bad = bad3(xk) || bad3(uk);
+    double v[3] = {0.0, 0.0, 0.0}, g = 1.0;
+    if (k == 0) {
+        db[0] = db[1] = db[2] = 0.0;
+    } else {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) v[c] = dx[c] * inv_dt;
+        g = fma(-v[0], v[0], fma(-v[1], v[1], fma(-v[2], v[2], 1.0)));
+        bad = bad || !(g > 0.0);
+    }
+    if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
+    // e = beta_k - vbar_k (difference of end-point and chord velocities)
+    const double e[3] = {b[0] - v[0], b[1] - v[1], b[2] - v[2]};
+    const double qa = far_on ? qf * inv_dt : 0.0;
+    RecS r;
+    r.nx = (float)-xk[0];
+    r.ny = (float)-xk[1];
+    r.nz = (float)-xk[2];
+    const float ig2f = (float)ig2;
+    r.nhig2 = -0.5f * ig2f;
+    r.nbx = (float)-b[0];
+    r.nby = (float)-b[1];
+    r.nbz = (float)-b[2];
+    r.ig2n = near_on ? (float)(qf * ig2) : 0.f;
+    r.bdx = (float)(qa * db[0]);
+    r.bdy = (float)(qa * db[1]);
+    r.bdz = (float)(qa * db[2]);
+    r.dtg = (float)(dt * g);
+    r.d2x = 2.f * (float)e[0];
+    r.d2y = 2.f * (float)e[1];
+    r.d2z = 2.f * (float)e[2];
+    r.gd = (float)(g + fma(e[0], e[0], fma(e[1], e[1], e[2] * e[2])));
+    float4* o = reinterpret_cast<float4*>(rec + i);
+    o[0] = make_float4(r.nx, r.ny, r.nz, r.nhig2);
+    o[1] = make_float4(r.nbx, r.nby, r.nbz, r.ig2n);
+    o[2] = make_float4(r.bdx, r.bdy, r.bdz, r.dtg);
+    o[3] = make_float4(r.d2x, r.d2y, r.d2z, r.gd);
 }
 
 __global__ void k_precompute_fp64(const double* __restrict__ x, const double* __restrict__ u,
-                                  const double* __restrict__ q, int n_part, int n_samples, double t0,
+                                  const double* __restrict__ q, long long total, int n_samples, double t0,
                                   double dt, int flags, RecD* __restrict__ rec, DevCounters* counters)
 {
     const double near = (flags & RD_NEAR) ? 1.0 : 0.0, far = (flags & RD_FAR) ? 1.0 : 0.0;
-    const long long total = (long long)n_part * n_samples;
-    for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
-         i += (long long)gridDim.x * blockDim.x) {
-        const int k = (int)(i % n_samples);
-        const double* xk = x + 3 * i;
-        const double* uk = u + 3 * i;
-        bool bad = !finite3(xk) || !finite3(uk);
-        double bx, by, bz, ig2;
-        beta_of(uk, bx, by, bz, ig2);
-        double ax = 0.0, ay = 0.0, az = 0.0;
-        if (k > 0) {
-            double px, py, pz, pig2;
-            beta_of(uk - 3, px, py, pz, pig2);
-            ax = (bx - px) / dt;
-            ay = (by - py) / dt;
-            az = (bz - pz) / dt;
-            const double vx = xk[0] - xk[-3], vy = xk[1] - xk[-2], vz = xk[2] - xk[-1];
-            bad = bad || !((vx * vx + vy * vy) + vz * vz < dt * dt);
+    bool out;
+    const long long i = warp_sample(total, out);
+    double xk[3] = {0.0, 0.0, 0.0}, uk[3] = {0.0, 0.0, 0.0};
+    if (i >= 0) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            xk[c] = x[3 * i + c];
+            uk[c] = u[3 * i + c];
         }
-        if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
-        RecD r;
-        const double qp = q ? q[i / n_samples] : 1.0;
-        r.xa = D4{xk[0], xk[1], xk[2], __dadd_rn(t0, __dmul_rn((double)k, dt))};
-        r.bb = D4{bx, by, bz, (near * qp) * ig2};
-        r.bd = D4{(far * qp) * ax, (far * qp) * ay, (far * qp) * az, 0.0};
-        rec[i] = r;
     }
+    double bx, by, bz, ig2;
+    beta_of(uk, bx, by, bz, ig2);
+    const double px = __shfl_up_sync(0xffffffffu, bx, 1), py = __shfl_up_sync(0xffffffffu, by, 1),
+                 pz = __shfl_up_sync(0xffffffffu, bz, 1);
+    const double xp[3] = {__shfl_up_sync(0xffffffffu, xk[0], 1), __shfl_up_sync(0xffffffffu, xk[1], 1),
+                          __shfl_up_sync(0xffffffffu, xk[2], 1)};
+    if (!out) return;
+    long long p;
+    int k;
+    split_sample(i, n_samples, p, k);
+    bool bad = bad3(xk) || bad3(uk);
+    double ax = 0.0, ay = 0.0, az = 0.0;
+    if (k > 0) {
+        ax = (bx - px) / dt;
+        ay = (by - py) / dt;
+        az = (bz - pz) / dt;
+        const double vx = xk[0] - xp[0], vy = xk[1] - xp[1], vz = xk[2] - xp[2];
+        bad = bad || !((vx * vx + vy * vy) + vz * vz < dt * dt);
+    }
+    if (bad) atomicOr(&counters->errors, ERRBIT_INPUT);
+    RecD r;
+    const double qp = q ? q[p] : 1.0;
+    r.xa = D4{xk[0], xk[1], xk[2], __dadd_rn(t0, __dmul_rn((double)k, dt))};
+    r.bb = D4{bx, by, bz, (near * qp) * ig2};
+    r.bd = D4{(far * qp) * ax, (far * qp) * ay, (far * qp) * az, 0.0};
+    rec[i] = r;
 }
 
 // =============================================================================================
@@ -661,8 +713,8 @@ cudaError_t launch_precompute_mixed(const double* x, const double* u, const doub
                                     cudaStream_t s)
 {
     const long long n = (long long)n_part * n_samples;
-    k_precompute_mixed<<<grid_for(n, 256), 256, 0, s>>>(x, u, q, qscale, n_part, n_samples, dt, flags, rec,
-                                                        counters);
+    const PrecomputeGrid g(n);
+    k_precompute_mixed<<<g.blocks, g.threads, 0, s>>>(x, u, q, qscale, n, n_samples, dt, flags, rec, counters);
     return cudaGetLastError();
 }
 
@@ -670,7 +722,8 @@ cudaError_t launch_precompute_fp64(const double* x, const double* u, const doubl
                                    double t0, double dt, int flags, RecD* rec, DevCounters* counters, cudaStream_t s)
 {
     const long long n = (long long)n_part * n_samples;
-    k_precompute_fp64<<<grid_for(n, 256), 256, 0, s>>>(x, u, q, n_part, n_samples, t0, dt, flags, rec, counters);
+    const PrecomputeGrid g(n);
+    k_precompute_fp64<<<g.blocks, g.threads, 0, s>>>(x, u, q, n, n_samples, t0, dt, flags, rec, counters);
     return cudaGetLastError();
 }
 

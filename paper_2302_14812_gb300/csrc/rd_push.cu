@@ -59,7 +59,11 @@ cudaError_t launch_push_boris(int n_part, int n_steps, double dt, const double* 
                               double* x_out, double* u_out, cudaStream_t s)
 {
     if (n_part <= 0 || n_steps <= 0) return cudaSuccess;
-    k_push_boris<<<(n_part + 127) / 128, 128, 0, s>>>(n_part, n_steps, dt, B[0], B[1], B[2], qm, x, u, x_out, u_out);
+    // one-warp CTAs while they do not fill the multiprocessors: the warps of a CTA share one SM's FP64 pipe
+    // (256 particles x 25 steps: 24 us in two CTAs of 128 threads, 9 us in eight of 32)
+    const int threads = n_part <= 4 * 32 * sm_count() ? 32 : 128;
+    k_push_boris<<<(n_part + threads - 1) / threads, threads, 0, s>>>(n_part, n_steps, dt, B[0], B[1], B[2], qm, x, u,
+                                                                      x_out, u_out);
     return cudaGetLastError();
 }
 
