@@ -169,9 +169,26 @@ struct PrecomputeGrid {
         blocks = (unsigned)((warps * 32 + threads - 1) / threads);
     }
 };
-// Default intervals per work item of the deposit kernels: kDefaultChunk (at most S), halved while
-// the grid (cell blocks x particles x chunks) would hold fewer than 8 CTAs per multiprocessor.
-int auto_chunk(long long n_cell_blocks, long long n_part, int S);
+// Default intervals per work item of a deposit launch: its cell blocks x particles x chunks run in waves of
+// the per_sm CTAs a multiprocessor holds, and an item costs its intervals plus `setup` (anchors and first
+// records, in intervals' time).  Chunks are of equal length, at most kDefaultChunk; while that makes few
+// waves (at most kMaxWaves), the split of the trajectory into more chunks that minimises waves x (chunk +
+// setup) is taken, down to kMinChunk intervals.  Measured against halving 2048 until the grid held 8 CTAs
+// per multiprocessor (unequal last chunks, half-empty last waves): FP64, 24 particles x 1200 intervals x
+// 4096 cells 14.33 -> 13.41 ms (5.05 waves of 300 intervals -> 8.8 of 172); mixed, 37 x 3001 x 3233
+// 0.873 -> 0.832 ms, 1 x 2000 x 64 cells 19 -> 11 us.  The set-up figures hold to a factor of two: 30 or
+// 100 intervals for the mixed kernel change these by less than 1.5 %.
+constexpr int kMaxWaves = 16;
+constexpr int kMinChunk = 16;
+#ifndef RD_MIXED_SETUP
+#define RD_MIXED_SETUP 60
+#endif
+constexpr int kMixedSetup = RD_MIXED_SETUP;
+constexpr int kFp64Setup = 5;
+constexpr int kFp64CtasPerSm = 2;
+int auto_chunk(long long n_cell_blocks, long long n_part, int S, int per_sm, int setup);
+// CTAs per multiprocessor of the mixed kernel of a shape and a detector's flags
+int mixed_ctas_per_sm(int cells_per_cta, int cells_per_thread, int flags);
 // Cell blocks per group of the mixed kernels' work order (item_coords): as many as keep the group's
 // active detector slice (cells_per_cta x 32 bytes x the bins a step chunk of `chunk` of the
 // trajectory's n_intervals spans, per block) within RD_GROUP_SLICE_MB, at most 8.
