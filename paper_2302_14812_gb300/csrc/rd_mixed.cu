@@ -223,36 +223,6 @@ __device__ __forceinline__ void field_at_ff(const RecS& r, float nx, float ny, f
     o.rinv = 1.f;
 }
 
-// Interval of cell j that passes two or more bin edges (rare): flush the bin being filled and the
-// whole bins inside the interval, leaving the state one edge short so that the common path below
-// finishes the step (it flushes the last whole bin and starts the next).
-template <int NC, int NT, bool TRACK, bool FF>
-__device__ __forceinline__ void multi_edges(Cells<NC>& c, const Cold<NC, NT>& cold, int j, const Field& o,
-                                            const Consts& C, float& fn, int k, int k_begin, int k_end)
-{
-    const float f = fn;
-    if (!(f >= 2.f * C.W)) return;
-    const int rb = row_base<NT>(j, C.n_bins), b0 = c.bo[j] - rb;
-    const int m = (int)fminf(floorf(f * C.invW), 16777216.f);      // edges passed, >= 2
-    flush_acc<NC, FF>(C, c, j, b0, c.bo[j]);
-    const float fs = C.W * o.S, fb = fs * o.rinv;
-    // whole bins b0+1 .. b0+m-2 now; bin b0+m-1 is left in the accumulator for the common path
-    const int lo = max(b0 + 1, 0), hi = min(b0 + m - 2, C.n_bins - 1);
-    for (int b = lo; b <= hi; ++b)
-        flush(C, b, rb + b, o.E[0] * fs, o.E[1] * fs, o.E[2] * fs, o.B[0] * fb, o.B[1] * fb, o.B[2] * fb);
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        c.acc[i][j] = o.E[i] * fs;
-        if (!FF) c.acc[3 + i][j] = o.B[i] * fb;
-    }
-    c.bo[j] += m - 1;
-    fn = fminf(fmaxf(fmaf(-(float)(m - 1), C.W, f), C.W), C.W * 1.99999988f);
-    if (TRACK) {
-        if (b0 < 0 && b0 + m - 1 >= 0) cold.set(j, kBelow, k - k_begin + 1);
-        if (b0 < C.n_bins && b0 + m - 1 >= C.n_bins) cold.set(j, kAbove, k_end - k + 1);
-    }
-}
-
 // Field of the sample in bin-weight units per unit dt: G = (S E', (S/R) d x E').
 __device__ __forceinline__ void scaled_field(const Field& o, float* G)
 {
@@ -328,7 +298,8 @@ __device__ __forceinline__ void multi_edges_lin(Cells<NC>& c, const Cold<NC, NT>
 // edges; such an interval sets the cell's time to -inf, after which the cell crosses no edge and
 // flushes nothing for the rest of the tile.  kExact: the same arithmetic plus the multi-edge case;
 // used to walk a tile again (from its saved start) for a warp in which some cell stopped, flushing
-// only from the interval that stopped it onwards (earlier bins were flushed by the fast walk).
+// only from the interval that stopped it onwards (earlier bins were flushed by the fast walk), and to
+// walk that warp's next tile at once.  Held field: exact_tile; step's kExact: interpolated fields.
 // Both walks evaluate every value with the same operations in the same order (no implicit
 // contraction), so they agree bit for bit up to that interval.
 enum { kFast = 0, kExact = 1 };
@@ -340,7 +311,7 @@ enum { kFast = 0, kExact = 1 };
 // counted).  ok: kExact only, false from the interval that stopped the fast walk onwards.
 template <int NC, int NT, int MODE, bool LAST, bool TRACK, bool FF, int LIN>
 __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& C, const Cold<NC, NT>& cold, int k,
-                                     int k_begin, int k_end, bool* ok, float ramp)
+                                     int k_begin, int k_end, bool* ok, float ramp, bool again = false)
 {
     constexpr int NF = FF ? 3 : 6;                  // carried field components (far field: E only)
     constexpr bool QUAD = LIN == 2;                 // quadratic interpolation (RD_QUADRATIC)
@@ -404,11 +375,8 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
     if (MODE == kExact) {
 #pragma unroll
         for (int j = 0; j < NC; ++j) {
-            if (LIN)
-                multi_edges_lin<NC, NT, TRACK, FF, QUAD>(c, cold, j, G[j], D2[j], L[j], inv2L[j], C, fn[j], k, k_begin,
-                                                         k_end);
-            else
-                multi_edges<NC, NT, TRACK, FF>(c, cold, j, o[j], C, fn[j], k, k_begin, k_end);
+            multi_edges_lin<NC, NT, TRACK, FF, QUAD>(c, cold, j, G[j], D2[j], L[j], inv2L[j], C, fn[j], k, k_begin,
+                                                     k_end);
         }
     }
 #pragma unroll
@@ -452,7 +420,7 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
             }
         } else {
             const int b = TRACK || RD_CHECK ? c.bo[j] - row_base<NT>(j, C.n_bins) : 0;
-            const bool go = MODE == kFast || !ok[j];
+            const bool go = MODE == kFast || !(again && ok[j]);
             const bool pr = cr && go && (TRACK ? (unsigned)b < (unsigned)C.n_bins : (!RD_CHECK || bin_ok(C, b)));
             float* a = bin_addr(C, c.bo[j]);
             const float e[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
@@ -725,13 +693,18 @@ __device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, cons
     }
 }
 
-// Per-thread copy of the walk state at the start of a tile, in shared memory ([word][thread]):
-// f, rpd, bo, below, above, acc[6], gp[6], and for the quadratic interpolation gpp[6], hp.
+// Scratch of a warp in shared memory: save_cell words for each of its 32 NC cells.  The fast walk keeps
+// the state at the start of a tile there ([word][lane]: f, rpd, bo, below, above, acc[6], gp[6], and for
+// the quadratic interpolation gpp[6], hp); the exact walk, once it has taken that state back, hands its
+// runs of finished bins over there (add_runs: 16 words per lane).
 constexpr int save_cell(int lin) { return lin == 2 ? 24 : 17; }
 
+
 template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT>& cold, float (*sv)[NT], int tid)
+__device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT>& cold, float* scratch)
 {
+    float (*sv)[32] = reinterpret_cast<float (*)[32]>(scratch);
+    const int tid = threadIdx.x & 31;
     constexpr int NF = FF ? 3 : 6;
     constexpr int kSaveCell = save_cell(LIN);
 #pragma unroll
@@ -758,8 +731,10 @@ __device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT
 }
 
 template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& cold, float (*sv)[NT], int tid)
+__device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& cold, const float* scratch)
 {
+    const float (*sv)[32] = reinterpret_cast<const float (*)[32]>(scratch);
+    const int tid = threadIdx.x & 31;
     constexpr int NF = FF ? 3 : 6;
     constexpr int kSaveCell = save_cell(LIN);
 #pragma unroll
@@ -785,15 +760,165 @@ __device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& 
     }
 }
 
-template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void walk_tile(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
-                                          float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
-                                          float (*sv)[NT])
+// ---------------------------------------------------------------------------------------------
+// Exact walk of the held field: any number of bin edges per interval.
+//
+// Where intervals pass several edges the walk is bound by the reductions: with a lane per cell every
+// finished bin is two reductions that share a 128-byte line with no other lane's, which L2 takes at
+// 9.2e10 bins/s (5e10 where the detector does not fit it).  Eight lanes adding four consecutive bins of
+// one cell with one instruction reach 1.5e11 (8e10; reductions alone, measured).  So where a cell of the
+// warp finishes kRunBins bins or more in a step, every lane hands its run over through shared memory and
+// groups of eight lanes add the runs.  Measured, deposit kernel, with the exact walk taken at once where
+// the tile before needed it (before: fast walk, then exact walk lane by lane): one electron, 38000 steps
+// x 512 cells x 131072 bins (3.4 edges a step) 2.17 -> 1.12 ms; 400 steps x 4096 cells x 8192 bins (20 a
+// step) 0.322 -> 0.261 ms; 256 electrons x 1200 cells, 25 steps a call (2 a step) 0.195 -> 0.178 ms.
+// Gathering whole 128-byte lines of four bins per cell before adding them cost more instructions than
+// the fuller lines saved (1.09, 0.338, 0.226 ms).
+// ---------------------------------------------------------------------------------------------
+// Shortest run, of any cell of the warp, that is handed over; 2, 4 and 6 on the cases above: 0.98, 1.21 and
+// 1.61 ms; 0.260, 0.264 and 0.262 ms; 0.216, 0.205 and 0.212 ms.
+constexpr int kRunBins = 3;
+// Lane's run: `count` consecutive bins from bin b of cell row j's detector row; bin 0 is `e0`, `h0` (E and
+// B) if `first`, every other one `e1`, `h1`.  Called by the converged warp; stage: 32 x 4 float4 of the warp.
+template <int NT>
+__device__ __forceinline__ void add_runs(const Consts& C, float4* stage, int j, int b, int count, bool first,
+                                         const float* e0, const float* h0, const float* e1, const float* h1)
 {
-    const int tid = threadIdx.x;
+    const int lane = threadIdx.x & 31;
+    // chunk c of a lane, XORed so that eight lanes' 16-byte stores fall on distinct banks
+    auto chunk = [&](int l, int c) -> float4& { return stage[l * 4 + (c ^ ((l >> 1) & 3))]; };
+    __syncwarp();
+    chunk(lane, 0) = make_float4(e0[0], e0[1], e0[2], h0[0]);
+    chunk(lane, 1) = make_float4(h0[1], h0[2], 0.f, 0.f);
+    chunk(lane, 2) = make_float4(e1[0], e1[1], e1[2], h1[0]);
+    chunk(lane, 3) = make_float4(h1[1], h1[2], 0.f, 0.f);
+    __syncwarp();
+    const int group = lane >> 3, sub = (lane >> 1) & 3, half = lane & 1;
+    const int info = count * 2 + (first ? 1 : 0);
+    const int row0 = (j * NT + (int)(threadIdx.x & ~31u) + group) * C.n_bins + sub;
+    for (int i0 = 0; __any_sync(0xffffffffu, i0 < count); i0 += 4) {
+        const int i = i0 + sub;
+#pragma unroll 4
+        for (int g = 0; g < 8; ++g) {
+            const int owner = 4 * g + group;
+            const int ob = __shfl_sync(0xffffffffu, b, owner), oi = __shfl_sync(0xffffffffu, info, owner);
+            if (2 * i < (oi & ~1)) {
+                const float4 v = chunk(owner, (i == 0 && (oi & 1) ? 0 : 2) + half);
+                red_add_v4(bin_addr(C, row0 + 4 * g * C.n_bins + ob + i0) + 4 * half, v.x, v.y, v.z, v.w);
+            }
+        }
+    }
+}
+
+template <int NC, int NT, bool FF>
+__device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
+                                           const Cold<NC, NT>& cold, int k0, int k_begin, int k_end, float* scratch,
+                                           bool again, bool track)
+{
+    bool ok[NC];                    // no interval of two or more edges so far
+#pragma unroll
+    for (int j = 0; j < NC; ++j) ok[j] = true;
+#pragma unroll 1
+    for (int i = 0; i < cnt; ++i) {
+        const RecS& r = tile[i];
+        const bool last = last_tile && i == cnt - 1;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) {
+            Field o;
+            if (FF)
+                field_at_ff(r, c.px[j], c.py[j], c.pz[j], c.rpd[j], c.nlx[j], c.nly[j], c.nlz[j], o);
+            else
+                field_at(r, c.px[j], c.py[j], c.pz[j], c.rpd[j], C, o);
+            const float t = last ? fmaf((float)(cold.bo_end(j) - c.bo[j]), C.W, cold.f_end(j))
+                                 : fmaf(o.num, o.rden, c.f[j]);
+            const float ws = (fminf(t, C.W) - c.f[j]) * o.S, wb = FF ? ws : ws * o.rinv;
+#pragma unroll
+            for (int q = 0; q < 3; ++q) {
+                c.acc[q][j] = fmaf(o.E[q], ws, c.acc[q][j]);
+                if (!FF) c.acc[3 + q][j] = fmaf(o.B[q], wb, c.acc[3 + q][j]);
+            }
+            // edges passed, and the time left in the last bin
+            ok[j] = ok[j] && t < 2.f * C.W;
+            int m = t >= C.W ? 1 : 0;
+            float rem = t - C.W;
+            if (t >= 2.f * C.W) {
+                m = max(2, (int)fminf(floorf(t * C.invW), 16777216.f));
+                rem = fminf(fmaxf(fmaf(-(float)m, C.W, t), 0.f), C.W * 0.99999994f);
+            }
+            // finished bins b0 .. b0 + m - 1, those inside the window: the first from the accumulator, the
+            // others whole bins of this interval's field
+            const int b0 = c.bo[j] - row_base<NT>(j, C.n_bins);
+            const int b = max(b0, 0);
+            const int count = again && ok[j] ? 0 : max(0, min(b0 + m, C.n_bins) - b);
+            if (__any_sync(0xffffffffu, count > 0)) {
+                const bool first = b == b0;         // false: the window starts inside the interval
+                const int rest = count - (first ? 1 : 0);
+                const float e0[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
+                const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
+                float h0[3], e1[3], h1[3];
+                bin_b<NC, FF>(c, j, e0, cb, h0);
+                const bool runs = __any_sync(0xffffffffu, count >= kRunBins);
+                if (!runs && first && count > 0) {
+                    float* a = bin_addr(C, c.bo[j]);
+                    red_add_v4(a, e0[0], e0[1], e0[2], h0[0]);
+                    red_add_v2(a + 4, h0[1], h0[2]);
+                }
+                if (__any_sync(0xffffffffu, rest > 0)) {
+                    const float fs = C.W * o.S, fb = FF ? fs : fs * o.rinv;
+                    float cb1[3];
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        e1[q] = o.E[q] * fs;
+                        cb1[q] = FF ? 0.f : o.B[q] * fb;
+                    }
+                    bin_b<NC, FF>(c, j, e1, cb1, h1);
+                    if (runs) {
+                        add_runs<NT>(C, reinterpret_cast<float4*>(scratch), j, b, count, first, e0, h0, e1, h1);
+                    } else {
+                        float* a = bin_addr(C, row_base<NT>(j, C.n_bins) + b + (first ? 1 : 0));
+#pragma unroll
+                        for (int q = 0; q < kRunBins - 1; ++q) {
+                            if (q < rest) {
+                                red_add_v4(a + 8 * q, e1[0], e1[1], e1[2], h1[0]);
+                                red_add_v2(a + 8 * q + 4, h1[1], h1[2]);
+                            }
+                        }
+                    }
+                }
+            }
+            if (m > 0) {
+                const float rs = rem * o.S, rb = FF ? rs : rs * o.rinv;
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    c.acc[q][j] = o.E[q] * rs;
+                    if (!FF) c.acc[3 + q][j] = o.B[q] * rb;
+                }
+                if (track) {
+                    if (b0 < 0 && b0 + m >= 0) cold.set(j, kBelow, k0 + i - k_begin + 1);
+                    if (b0 < C.n_bins && b0 + m >= C.n_bins) cold.set(j, kAbove, k_end - (k0 + i) + 1);
+                }
+            }
+            c.f[j] = m > 0 ? rem : t;
+            c.bo[j] += m;
+        }
+    }
+    bool met = false;
+#pragma unroll
+    for (int j = 0; j < NC; ++j) met = met || !ok[j];
+    __syncwarp();                   // the scratch may hold saved states again
+    return __any_sync(0xffffffffu, met);
+}
+
+// The fast walk of one tile; false if it met an interval of two or more edges (the state is then back at the
+// tile's start).
+template <int NC, int NT, bool TRACK, bool FF, int LIN>
+__device__ __forceinline__ bool fast_tile(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
+                                          float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
+                                          float* scratch)
+{
     const int n_regular = last_tile ? cnt - 1 : cnt;
-    save_state<NC, NT, TRACK, FF, LIN>(c, cold, sv, tid);
     bool ok[NC];
+    save_state<NC, NT, TRACK, FF, LIN>(c, cold, scratch);
     if constexpr (NC == 2 && !TRACK && LIN == 0) {
         int i = 0;
 #pragma unroll 1
@@ -810,16 +935,34 @@ __device__ __forceinline__ void walk_tile(Cells<NC>& c, const RecS* tile, int cn
     bool stopped = false;
 #pragma unroll
     for (int j = 0; j < NC; ++j) stopped = stopped || c.f[j] == -INFINITY;
-    if (__any_sync(0xffffffffu, stopped)) {
-        // some interval of a cell of this warp passed two or more bin edges: walk the tile again
-        restore_state<NC, NT, TRACK, FF, LIN>(c, cold, sv, tid);
+    if (!__any_sync(0xffffffffu, stopped)) return true;
+    restore_state<NC, NT, TRACK, FF, LIN>(c, cold, scratch);
+    return false;
+}
+
+// The exact walk of one tile; again: after a fast walk that stopped (earlier bins are flushed).  Returns
+// whether the warp met an interval of two or more edges.
+template <int NC, int NT, bool FF, int LIN>
+__device__ __forceinline__ bool exact_walk(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
+                                           float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
+                                           float* scratch, bool again, bool track)
+{
+    if constexpr (LIN == 0) {
+        return exact_tile<NC, NT, FF>(c, tile, cnt, last_tile, C, cold, k0, k_begin, k_end, scratch, again, track);
+    } else {
+        const int n_regular = last_tile ? cnt - 1 : cnt;
+        bool ok[NC];
 #pragma unroll
         for (int j = 0; j < NC; ++j) ok[j] = true;
 #pragma unroll 1
         for (int i = 0; i < n_regular; ++i)
-            step<NC, NT, kExact, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
+            step<NC, NT, kExact, false, true, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp, again);
         if (last_tile)
-            step<NC, NT, kExact, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp);
+            step<NC, NT, kExact, true, true, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp, again);
+        bool met = false;
+#pragma unroll
+        for (int j = 0; j < NC; ++j) met = met || !ok[j];
+        return __any_sync(0xffffffffu, met);
     }
 }
 
@@ -831,8 +974,8 @@ __device__ __forceinline__ void walk_tile(Cells<NC>& c, const RecS* tile, int cn
 // Returns false if a bounded wait ran out (the error is recorded; the CTA must stop).
 template <bool FF, int LIN, int NC, int CPC>
 __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int cb, int ch,
-                                             RecS (*tile)[kTileSteps], uint64_t* bar, float (*sv)[CPC / NC],
-                                             unsigned& g_base)
+                                             RecS (*tile)[kTileSteps], uint64_t* bar, float (*cold_words)[CPC / NC],
+                                             float* scratch, unsigned& g_base)
 {
     constexpr int NT = CPC / NC;                // threads of the CTA
     const int S = P.n_samples - 1;
@@ -869,9 +1012,10 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
 
     // anchors: exact FP64 arrival (bins) at both ends of the chunk, per cell
     Cells<NC> c;
-    const Cold<NC, NT> cold{sv + NC * save_cell(LIN)};
+    const Cold<NC, NT> cold{cold_words};
+    scratch += (tid >> 5) * 32 * NC * save_cell(LIN);       // this warp's part
     float hp0[NC];                              // quadratic: length of interval k_begin - 1 (dt units)
-    bool partial = false;
+    bool partial = false, many = false;
     unsigned long long clip = 0, crossed = 0;
     const double* xp = P.x + (size_t)p * P.n_samples * 3;
 #pragma unroll
@@ -942,6 +1086,7 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
                 // drift by far less than a bin before the end anchor corrects it)
                 partial = partial || (ua < 1.0) || (ue > (double)P.n_bins - 1.0);
                 crossed += (unsigned long long)max(0, bo_end - c.bo[j]);
+                many = many || bo_end - c.bo[j] > n_int;
             }
         }
         cold.set(j, kBoEnd, bo_end);
@@ -990,6 +1135,7 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         }
     }
     const bool track = __syncthreads_or(partial) != 0;
+    many = __any_sync(0xffffffffu, many);
 
     for (int t = 0; t < n_tiles; ++t) {
         const unsigned g = g_base + t;
@@ -1008,12 +1154,18 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         const int k0 = k_begin + t * kTileSteps;
         const int cnt = min(kTileSteps, k_end - k0 + 1);
         const bool last_tile = (t == n_tiles - 1);
-        if (track)
-            walk_tile<NC, NT, true, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, cold, k0,
-                                          k_begin, k_end, sv);
-        else
-            walk_tile<NC, NT, false, FF, LIN>(c, tile[buf], cnt, last_tile, C, P.lin == 2 ? 0.f : 1.f, cold, k0,
-                                          k_begin, k_end, sv);
+        // many (warp-uniform): the warp's last tile met intervals of two or more edges (at the start: the
+        // anchors say more than one edge an interval), so this one goes to the exact walk at once
+        const float ramp = P.lin == 2 ? 0.f : 1.f;
+        bool done = false;
+        if (!many)
+            done = track ? fast_tile<NC, NT, true, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin,
+                                                            k_end, scratch)
+                         : fast_tile<NC, NT, false, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin,
+                                                             k_end, scratch);
+        if (!done)
+            many = exact_walk<NC, NT, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin, k_end, scratch,
+                                               !many, track);
         __syncthreads();
         if (tid == 0 && t + 2 < n_tiles) {
             fence_proxy_async();
@@ -1072,12 +1224,13 @@ __global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, FF, LIN))
     constexpr int NT = CPC / NC;
     __shared__ __align__(128) RecS tile[2][kTileSteps];
     __shared__ __align__(8) uint64_t bar[2];
-    __shared__ float sv[NC * (save_cell(LIN) + kColdWords)][NT];
+    __shared__ float cold[NC * kColdWords][NT];
+    __shared__ __align__(16) float scratch[CPC * save_cell(LIN)];
     init_staging(bar);
     int p, cb, ch;
     item_coords(blockIdx.x, P, p, cb, ch);
     unsigned g = 0;
-    (void)deposit_item<FF, LIN, NC, CPC>(P, p, cb, ch, tile, bar, sv, g);
+    (void)deposit_item<FF, LIN, NC, CPC>(P, p, cb, ch, tile, bar, cold, scratch, g);
 }
 
 // Persistent form: the resident CTAs draw work items of all problems from one counter.
@@ -1095,7 +1248,8 @@ __global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads,
     __shared__ __align__(128) RecS tile[2][kTileSteps];
     __shared__ __align__(8) uint64_t bar[2];
     __shared__ long long s_next;
-    __shared__ float sv[kMixedCells * (save_cell(LIN) + kColdWords)][kMixedThreads];
+    __shared__ float cold[kMixedCells * kColdWords][kMixedThreads];
+    __shared__ __align__(16) float scratch[kMixedCellsPerCta * save_cell(LIN)];
     init_staging(bar);
     const long long total = item_off[n_probs];
     unsigned g = 0;
@@ -1113,7 +1267,7 @@ __global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads,
         const DepositParams P = probs[lo];
         int p, cb, ch;
         item_coords((unsigned)(item - item_off[lo]), P, p, cb, ch);
-        if (!deposit_item<FF, LIN, kMixedCells, kMixedCellsPerCta>(P, p, cb, ch, tile, bar, sv, g)) break;
+        if (!deposit_item<FF, LIN, kMixedCells, kMixedCellsPerCta>(P, p, cb, ch, tile, bar, cold, scratch, g)) break;
     }
 }
 

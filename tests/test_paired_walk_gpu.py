@@ -4,7 +4,7 @@ The one-cell-per-thread shape walks the same operations one interval at a time, 
 step chunk adds every (cell, bin) once, so the two shapes must give the same FP32 fields, bit for bit.
 The bin widths (in steps) cover: two intervals that seldom pass an edge, that pass one in either
 interval, that pass one each (the single-step fallback), and intervals that pass several (the exact
-re-walk).  The lengths cover odd and even step counts around a 64-interval tile and its neighbours.
+walk).  The lengths cover odd and even step counts around a 64-interval tile and its neighbours.
 """
 import numpy as np
 import pytest
@@ -57,7 +57,7 @@ def _deposit(tr, det, nc=None):
     return E, B
 
 
-@pytest.mark.parametrize("width", [9.0, 2.3, 1.1, 0.45])
+@pytest.mark.parametrize("width", [9.0, 2.3, 1.1, 0.45, 0.1])
 @pytest.mark.parametrize("n_steps", [1, 2, 3, 63, 64, 65, 66, 130, 401])
 def test_paired_walk_equals_single_steps(n_steps, width):
     tr, det = _case(n_steps, width)
@@ -74,4 +74,26 @@ def test_paired_walk_in_the_far_field_limit(n_steps, width):
     tr, det = _case(n_steps, width, rd.RD_FAR | rd.RD_FARFIELD)
     E, B = _deposit(tr, det)
     Eo, Bo, _ = oracle.deposit(tr, det)
+    assert parity_err(E, Eo) <= 1e-4 and parity_err(B, Bo) <= 1e-4
+
+
+@pytest.mark.parametrize("flags", [rd.RD_NEAR | rd.RD_FAR, rd.RD_FAR | rd.RD_FARFIELD])
+@pytest.mark.parametrize("width", [0.45, 0.1, 0.03])
+@pytest.mark.parametrize("n_steps", [1, 65, 130])
+def test_runs_of_bins(n_steps, width, flags):
+    """Intervals of 1 to 60 bins: short runs lane by lane, long ones handed over to groups of lanes; whole
+    windows, and windows that begin and end inside runs (clipping)."""
+    tr, det = _case(n_steps, width, flags)
+    E, B = _deposit(tr, det)
+    Eo, Bo, _ = oracle.deposit(tr, det)
+    assert parity_err(E, Eo) <= 1e-4 and parity_err(B, Bo) <= 1e-4
+    cut = W.Detector(det.pix_pos, det.pix_t0 + 7.4 * det.dt_det, 0.0, det.dt_det, max(1, det.n_bins - 16), flags)
+    Eo, Bo, clipped = oracle.deposit(tr, cut)
+    import torch
+    d = rd.RadiationDetector.from_workload(cut, "mixed")
+    d.deposit(torch.from_numpy(tr.x).cuda(), torch.from_numpy(tr.u).cuda(), torch.from_numpy(tr.q).cuda(), tr.t0, tr.dt)
+    E, B = d.read()
+    st = d.stats()
+    d.close()
+    assert st.n_clipped == clipped and st.device_errors == 0
     assert parity_err(E, Eo) <= 1e-4 and parity_err(B, Bo) <= 1e-4
