@@ -230,8 +230,9 @@ RD_API rd_status rd_stream_reset(rd_detector* det);
  * k = 0..N/2, angular frequency w_k = 2 pi k / (N dt_det).  The bins are averages over dt_det,
  * so the spectrum of the underlying field is out / sinc^2(w dt_det / 2) below the Nyquist
  * frequency.  out: caller-owned device memory, float[n_pix][N/2 + 1].  FP32 FFT (relative error
- * ~1e-6 of the spectrum's norm).  Requires N a power of two (else RD_ERR_ARG); scratch of
- * 32 * n_pix * N bytes held by the detector.  Asynchronous on `stream`.
+ * ~1e-6 of the spectrum's norm).  Requires N a power of two (else RD_ERR_ARG).  Scratch held by the
+ * detector: none for N <= 8192, at most 64 MB or one cell's 12 N bytes for N <= 2^22, else 32 * n_pix * N
+ * bytes.  Asynchronous on `stream`.
  */
 RD_API rd_status rd_power_spectrum(rd_detector* det, int32_t which, float* out, rd_stream stream);
 

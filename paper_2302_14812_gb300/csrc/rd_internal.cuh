@@ -291,9 +291,12 @@ cudaError_t launch_write_fields(void* fields, int precision, int n_pix, int n_bi
 // power spectra (rd_spectrum.cu): twiddles exp(-2 pi i j / N), j < N/2, computed on the host
 void fill_twiddles(float2* host, int N);
 constexpr int kFusedMaxN = 8192;   // longest series transformed in shared memory (24.5 N bytes per CTA)
+constexpr int kSplitMaxN = 1 << 22;  // longest series transformed as columns, then rows
 bool spectrum_fused(int N);
-cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* z,
-                                  float2* y, const float2* tw, float scale, float* P, cudaStream_t s);
+int spectrum_twiddle_length(int N);               // twiddle table of a length-N series: exp(-2 pi i j / M), j < M / 2
+size_t spectrum_work_bytes(int n_pix, int N);
+cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* work,
+                                  const float2* tw, float scale, float* P, cudaStream_t s);
 
 // ---------------------------------------------------------------------------------------------
 // device helpers: mbarrier, bulk async copy, vector reductions

@@ -8,7 +8,9 @@
 // |Fz(k)|^2 = |Z2(k)|^2.  Twiddles exp(-2 pi i j / N) are computed in FP64 once per length.
 // N <= kFusedMaxN: one kernel reads a cell's bins, runs both FP32 radix-2 transforms in shared
 // memory and writes the cell's spectrum (the fields are read once, the spectrum written once).
-// Longer series: FP32 Stockham radix-2 passes over the whole batch, one launch per pass.
+// Longer series, up to kSplitMaxN: N = N1 N2, two kernels that read and write each element once (transforms
+// of length N1 over the columns, of length N2 over the rows).  Beyond that: FP32 Stockham radix-2 passes
+// over the whole batch, one launch per pass.
 #include <math.h>
 
 #include <algorithm>
@@ -323,6 +325,256 @@ cudaError_t launch_fused(const T* fields, int n_pix, int N, int c0, const float2
     }
 }
 
+// ---------------------------------------------------------------------------------------------
+// Long series: n = n1 N2 + n2, k = k1 + N1 k2,
+//   X[k1 + N1 k2] = sum_{n2} w_{N2}^{n2 k2} [ w_N^{n2 k1} sum_{n1} w_{N1}^{n1 k1} x[n1 N2 + n2] ].
+// k_split_columns forms the bracket Y[k1][n2] for C = 4096 / N1 neighbouring columns n2 per CTA (each row n1
+// of them is C consecutive bins), k_split_rows the sums over n2 for rows k1 and N1 - k1, which hold the
+// frequencies k and N - k that the power of Z1 = F_x + i F_y needs together; Z2 = F_z is real, so its rows
+// k1 <= N1 / 2 suffice.  Bound by memory: 32 bytes read per bin and cell (whole sectors), 12 written and
+// read again for Y, 2 written for the power.  Cells go through both kernels in batches whose Y fits L2, so
+// only the bins and the power touch DRAM.  Measured, 512 cells x 131072 bins: 6.12 ms as 17 radix-2 passes
+// over the batch (4.3 GB each) plus packing and power; 0.90 ms in two kernels per batch of 42 cells (columns
+// 0.52 ms, 4.1 TB/s of the bins; rows 0.38 ms).
+// ---------------------------------------------------------------------------------------------
+constexpr int kColumnElems = 4096;      // elements of each of Z1, Z2 per CTA of k_split_columns, 16 per thread
+constexpr int kColumnThreads = kColumnElems / 16;
+
+// One Stockham pass (see spec_pass) of radix R at stride S over the columns of both transforms, rows of
+// C elements in shared memory (row i at pad(i)); LAST: the results go to global memory, multiplied by
+// exp(-2 pi i n2 k1 / N).  tw: exp(-2 pi i j / N1), j < N1 / 2.
+template <int N1, int S, typename T, int STRIDE>
+__device__ __forceinline__ void column_passes(float2* z1, float2* z2, const float2* tw, const T* row, int c0, int N2,
+                                              int n2, float two_over_n, float2* Y1, float2* Y2)
+{
+    constexpr int C = kColumnElems / N1, R = N1 / S >= 16 ? 16 : N1 / S, NB = 16 / R;
+    constexpr int n = N1 / S, m = n / R;
+    constexpr bool LAST = S * R == N1;
+    const int c = threadIdx.x % C, t = threadIdx.x / C;
+    float2 a1[NB][R], a2[NB][R];
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        const int b = t + u * (N1 / 16), q = b % S, p = b / S;
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+            const int i = q + S * (p + r * m);
+            if (S == 1) {
+                const float3 v = Load3<T, STRIDE>::get(row, i * N2 + n2, c0);
+                a1[u][r] = make_float2(v.x, v.y);
+                a2[u][r] = make_float2(v.z, 0.f);
+            } else {
+                a1[u][r] = z1[pad(i) * C + c];
+                a2[u][r] = z2[pad(i) * C + c];
+            }
+        }
+    }
+    if (S > 1) __syncthreads();         // every read of the pass is done
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        const int b = t + u * (N1 / 16), q = b % S, p = b / S;
+        dft_bitrev<R>(a1[u]);
+        dft_bitrev<R>(a2[u]);
+        const int o = q + S * R * p;
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            float2 b1 = a1[u][bitrev<R>(k)], b2 = a2[u][bitrev<R>(k)];
+            const int i = o + S * k;
+            if (LAST) {                 // m = 1, p = 0: no twiddle of its own; i = k1
+                float sn, cs;
+                sincospif(two_over_n * (float)(i * n2), &sn, &cs);      // exact argument: i n2 < N <= 2^22
+                const float2 w = make_float2(cs, -sn);
+                Y1[(size_t)i * N2 + n2] = cmul(b1, w);
+                if (i <= N1 / 2) Y2[(size_t)i * N2 + n2] = cmul(b2, w);
+            } else {
+                if (k > 0) {
+                    const float2 w = twiddle(tw, p * k * S, N1 / 2);
+                    b1 = cmul(b1, w);
+                    b2 = cmul(b2, w);
+                }
+                z1[pad(i) * C + c] = b1;
+                z2[pad(i) * C + c] = b2;
+            }
+        }
+    }
+    if constexpr (!LAST) {
+        __syncthreads();
+        column_passes<N1, S * R, T, STRIDE>(z1, z2, tw, row, c0, N2, n2, two_over_n, Y1, Y2);
+    }
+}
+
+constexpr size_t split_columns_smem(int N1)
+{
+    return sizeof(float2) * (2 * (size_t)(N1 + N1 / 16) * (kColumnElems / N1) + N1 / 2);
+}
+
+// grid (N2 / C, cells); tab: exp(-2 pi i j / M), j < M / 2, M = N1 tab_step
+template <int N1, typename T, int STRIDE>
+__global__ void __launch_bounds__(kColumnThreads, 2) k_split_columns(const T* __restrict__ fields, int c0, int N2,
+                                                                     const float2* __restrict__ tab, int tab_step,
+                                                                     float2* __restrict__ Y1, float2* __restrict__ Y2)
+{
+    extern __shared__ float2 sm[];
+    constexpr int C = kColumnElems / N1, zlen = (N1 + N1 / 16) * C;
+    float2* tw = sm + 2 * zlen;
+    for (int j = threadIdx.x; j < N1 / 2; j += kColumnThreads) tw[j] = tab[j * tab_step];
+    __syncthreads();
+    const size_t cell = blockIdx.y;
+    const int n2 = blockIdx.x * C + threadIdx.x % C;
+    const size_t N = (size_t)N1 * N2;
+    column_passes<N1, 1, T, STRIDE>(sm, sm + zlen, tw, fields + cell * N * STRIDE, c0, N2, n2, 2.f / (float)N,
+                                    Y1 + cell * N, Y2 + cell * (size_t)(N1 / 2 + 1) * N2);
+}
+
+// Rows: one Stockham pass over the three rows (Z1 at k1 and N1 - k1, Z2 at k1) of a row pair.
+template <int N2, int S>
+__device__ __forceinline__ void row_passes(float2* const (&z)[3], const float2* const (&src)[3], const float2* tw,
+                                           int t)
+{
+    constexpr int R = N2 / S >= 16 ? 16 : N2 / S, NB = 16 / R, m = N2 / S / R;
+    float2 a[3][NB][R];
+#pragma unroll
+    for (int v = 0; v < 3; ++v)
+#pragma unroll
+        for (int u = 0; u < NB; ++u) {
+            const int b = t + u * (N2 / 16), q = b % S, p = b / S;
+#pragma unroll
+            for (int r = 0; r < R; ++r) {
+                const int i = q + S * (p + r * m);
+                a[v][u][r] = S == 1 ? __ldg(src[v] + i) : z[v][pad(i)];
+            }
+        }
+    __syncthreads();                    // every read of the pass is done (first pass: tw is filled)
+#pragma unroll
+    for (int u = 0; u < NB; ++u) {
+        const int b = t + u * (N2 / 16), q = b % S, p = b / S;
+        const int o = q + S * R * p;
+#pragma unroll
+        for (int v = 0; v < 3; ++v) dft_bitrev<R>(a[v][u]);
+#pragma unroll
+        for (int k = 0; k < R; ++k) {
+            const float2 w = (m > 1 && k > 0) ? twiddle(tw, p * k * S, N2 / 2) : make_float2(1.f, 0.f);
+#pragma unroll
+            for (int v = 0; v < 3; ++v) {
+                const float2 x = a[v][u][bitrev<R>(k)];
+                z[v][pad(o + S * k)] = (m > 1 && k > 0) ? cmul(x, w) : x;
+            }
+        }
+    }
+    __syncthreads();
+    if constexpr (S * R < N2) row_passes<N2, S * R>(z, src, tw, t);
+}
+
+constexpr int row_pairs(int N2) { return N2 >= 4096 ? 1 : 4096 / N2; }          // per CTA
+constexpr int row_threads(int N2) { return row_pairs(N2) * (N2 / 16); }
+// row stride in shared memory: 16 bytes beyond a multiple of 128, so that neighbouring rows' elements at
+// one index (the power step) lie on different banks
+constexpr int row_stride(int N2) { return N2 + N2 / 16 + 2; }
+constexpr size_t split_rows_smem(int N2)
+{
+    return sizeof(float2) * (3 * (size_t)row_pairs(N2) * row_stride(N2) + N2 / 2);
+}
+
+// grid (ceil((N1 / 2 + 1) / row_pairs), cells)
+template <int N2>
+__global__ void __launch_bounds__(row_threads(N2), N2 <= 2048 ? 2 : 1)
+    k_split_rows(const float2* __restrict__ Y1, const float2* __restrict__ Y2, int N1, const float2* __restrict__ tab,
+                 int tab_step, float scale, float* __restrict__ P)
+{
+    extern __shared__ float2 sm[];
+    constexpr int G = row_pairs(N2), TT = N2 / 16, LD = row_stride(N2);
+    float2* tw = sm + 3 * G * LD;
+    for (int j = threadIdx.x; j < N2 / 2; j += row_threads(N2)) tw[j] = tab[j * tab_step];
+    const size_t N = (size_t)N1 * N2, cell = blockIdx.y;
+    const int first = blockIdx.x * G, half = N1 / 2;
+    const int g = threadIdx.x / TT, t = threadIdx.x % TT;
+    const int k1 = min(first + g, half);                // (a surplus row pair repeats the last)
+    const float2* const src[3] = {Y1 + cell * N + (size_t)k1 * N2, Y1 + cell * N + (size_t)((N1 - k1) % N1) * N2,
+                                  Y2 + (cell * (half + 1) + k1) * N2};
+    float2* const z[3] = {sm + (3 * g) * LD, sm + (3 * g + 1) * LD, sm + (3 * g + 2) * LD};
+    row_passes<N2, 1>(z, src, tw, t);
+    float* out = P + cell * (N / 2 + 1);
+    for (int e = threadIdx.x; e < G * N2; e += row_threads(N2)) {
+        const int h = e % G, k2 = e / G, kk = first + h;
+        if (kk > half) continue;
+        const float2* zr = sm + 3 * h * LD;
+        // N - k: row N1 - k1, element N2 - 1 - k2 (row 0: N2 - k2)
+        const int mir = kk == 0 ? (N2 - k2) & (N2 - 1) : N2 - 1 - k2;
+        const float2 a = zr[pad(k2)], b = zr[LD + pad(mir)], c = zr[2 * LD + pad(k2)];
+        const float pxy = 0.5f * (a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y);
+        const size_t k = (size_t)kk + (size_t)N1 * k2;
+        out[k <= N / 2 ? k : N - k] = scale * (pxy + (c.x * c.x + c.y * c.y));
+    }
+}
+
+int split_n2(int N) { return N <= 131072 ? 512 : std::min(4096, N / 256); }
+
+// cells per batch: their Y (12 bytes per bin and cell and a little more) within 64 MB of L2
+int split_batch(int n_pix, int N)
+{
+    const long long per_cell = 12LL * N + 8LL * split_n2(N);
+    return (int)std::max(1LL, std::min<long long>(n_pix, (64LL << 20) / per_cell));
+}
+
+template <int N1, typename T, int STRIDE>
+cudaError_t launch_columns(const T* fields, int cells, int c0, int N2, const float2* tab, int M, float2* Y1, float2* Y2,
+                           cudaStream_t s)
+{
+    auto k = k_split_columns<N1, T, STRIDE>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                               (int)split_columns_smem(N1));
+    if (e != cudaSuccess) return e;
+    k<<<dim3(N2 / (kColumnElems / N1), cells), kColumnThreads, split_columns_smem(N1), s>>>(fields, c0, N2, tab, M / N1,
+                                                                                           Y1, Y2);
+    return cudaGetLastError();
+}
+
+template <int N2>
+cudaError_t launch_rows(const float2* Y1, const float2* Y2, int cells, int N1, const float2* tab, int M, float scale,
+                        float* P, cudaStream_t s)
+{
+    auto k = k_split_rows<N2>;
+    const cudaError_t e = cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)split_rows_smem(N2));
+    if (e != cudaSuccess) return e;
+    const int pairs = N1 / 2 + 1, G = row_pairs(N2);
+    k<<<dim3((pairs + G - 1) / G, cells), row_threads(N2), split_rows_smem(N2), s>>>(Y1, Y2, N1, tab, M / N2, scale, P);
+    return cudaGetLastError();
+}
+
+template <typename T, int STRIDE>
+cudaError_t launch_split(const T* fields, int n_pix, int N, int c0, float2* work, const float2* tab, float scale, float* P,
+                         cudaStream_t s)
+{
+    const int N2 = split_n2(N), N1 = N / N2, M = std::max(N1, N2), batch = split_batch(n_pix, N);
+    float2* Y1 = work;
+    float2* Y2 = work + (size_t)batch * N;
+    for (int j = 0; j < n_pix; j += batch) {
+        const int cells = std::min(batch, n_pix - j);
+        const T* f = fields + (size_t)j * N * STRIDE;
+        float* out = P + (size_t)j * (N / 2 + 1);
+        cudaError_t e = cudaErrorInvalidValue;
+        switch (N1) {
+        case 32: e = launch_columns<32, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        case 64: e = launch_columns<64, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        case 128: e = launch_columns<128, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        case 256: e = launch_columns<256, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        case 512: e = launch_columns<512, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        case 1024: e = launch_columns<1024, T, STRIDE>(f, cells, c0, N2, tab, M, Y1, Y2, s); break;
+        default: break;
+        }
+        if (e != cudaSuccess) return e;
+        e = cudaErrorInvalidValue;
+        switch (N2) {
+        case 512: e = launch_rows<512>(Y1, Y2, cells, N1, tab, M, scale, out, s); break;
+        case 1024: e = launch_rows<1024>(Y1, Y2, cells, N1, tab, M, scale, out, s); break;
+        case 2048: e = launch_rows<2048>(Y1, Y2, cells, N1, tab, M, scale, out, s); break;
+        case 4096: e = launch_rows<4096>(Y1, Y2, cells, N1, tab, M, scale, out, s); break;
+        default: break;
+        }
+        if (e != cudaSuccess) return e;
+    }
+    return cudaSuccess;
+}
+
 int grid_for(long long n, int threads) { return grid_stride_blocks(n, threads, 32); }
 
 }  // namespace
@@ -337,11 +589,34 @@ void fill_twiddles(float2* host, int N)
 }
 
 bool spectrum_fused(int N) { return N >= 2 && N <= kFusedMaxN; }
+static bool spectrum_split(int N) { return N > kFusedMaxN && N <= kSplitMaxN; }
 
-// z: [2 n_pix][N] work array, y: same size (unused for N <= kFusedMaxN); tw: [N/2].
-cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* z,
-                                  float2* y, const float2* tw, float scale, float* P, cudaStream_t s)
+int spectrum_twiddle_length(int N)
 {
+    return spectrum_split(N) ? std::max(split_n2(N), N / split_n2(N)) : N;
+}
+
+size_t spectrum_work_bytes(int n_pix, int N)
+{
+    if (spectrum_fused(N)) return 0;
+    if (spectrum_split(N)) {
+        const size_t N2 = split_n2(N), N1 = N / N2;
+        return sizeof(float2) * (size_t)split_batch(n_pix, N) * ((size_t)N + (N1 / 2 + 1) * N2);
+    }
+    return 2 * sizeof(float2) * 2 * (size_t)n_pix * N;
+}
+
+// work: spectrum_work_bytes; tw: exp(-2 pi i j / M), j < M / 2, M = spectrum_twiddle_length(N).
+cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* work,
+                                  const float2* tw, float scale, float* P, cudaStream_t s)
+{
+    if (spectrum_split(N)) {
+        if (precision == RD_MIXED)
+            return launch_split<float, 8>(static_cast<const float*>(fields), n_pix, N, c0, work, tw, scale, P, s);
+        return launch_split<double, 6>(static_cast<const double*>(fields), n_pix, N, c0, work, tw, scale, P, s);
+    }
+    float2* z = work;                                   // two arrays [2 n_pix][N]
+    float2* y = work + 2 * (size_t)n_pix * N;
     if (spectrum_fused(N)) {
         if (precision == RD_MIXED)
             return launch_fused<float, 8>(static_cast<const float*>(fields), n_pix, N, c0, tw, scale, P, s);
