@@ -42,9 +42,6 @@ struct Cells {
     float rpd[NC];                  // R_{k-1} + dt (far-field limit: 1/R_c)
     float nlx[NC], nly[NC], nlz[NC];  // far-field limit: n_c - (its FP32 rounding in px, py, pz)
     float acc[6][NC];               // E xyz, B xyz of the current bin so far (weights in bins)
-    float gp[6][NC];                // linear / quadratic interpolation: scaled field of the previous sample
-    float gpp[6][NC];               // quadratic interpolation: scaled field two samples back ...
-    float hp[NC];                   // ... and the previous interval's length (units of dt)
     int bo[NC];                     // row * n_bins + bin being filled (bin may lie outside the window)
 };
 
@@ -223,104 +220,25 @@ __device__ __forceinline__ void field_at_ff(const RecS& r, float nx, float ny, f
     o.rinv = 1.f;
 }
 
-// Field of the sample in bin-weight units per unit dt: G = (S E', (S/R) d x E').
-__device__ __forceinline__ void scaled_field(const Field& o, float* G)
-{
-    const float sb = o.S * o.rinv;
-#pragma unroll
-    for (int i = 0; i < 3; ++i) {
-        G[i] = o.E[i] * o.S;
-        G[3 + i] = o.B[i] * sb;
-    }
-}
+// The walk of a tile.  The fast walk has no code for an interval that passes two or more bin edges; such an
+// interval sets the cell's time to -inf, after which the cell crosses no edge and flushes nothing for the
+// rest of the tile.  The exact walk handles any interval.  It walks a tile again (from its saved start)
+// for a warp in which some cell stopped, flushing only from the interval that stopped it onwards (earlier
+// bins were flushed by the fast walk), and then walks that warp's next tile at once.  Both evaluate the
+// arrival times with the same operations in the same order (no implicit contraction), so they agree bit
+// for bit up to that interval.
 
-// Linear interpolation (RD_LINEAR; with the ramp terms scaled to zero, ramp = 0, the previous field
-// held over the interval, RD_HOLD_PREV): over the interval the field goes linearly from G0 = gp (previous
-// sample) to G (this sample); the part [s0, s1] of the interval (dt units from its start, length L)
-// weighs G0 (s1 - s0) + (G - G0) (s1^2 - s0^2) / (2 L) = G0 (s1 - s0 - ramp) + G ramp with
-// ramp = (s1^2 - s0^2) / (2 L).  Quadratic interpolation (RD_QUADRATIC) adds D2 cu, D2 the second
-// divided difference of the scaled fields of samples k-2, k-1, k over their arrival times and
-// cu = int_{s0}^{s1} s (s - L) ds (qcube below).  Interval of cell j passing two or more bin
-// edges (exact walk only): flush the bin being filled, every whole bin, and leave the last, partial
-// bin in the accumulator with the time already in it; fn comes back below W (no edge left for the
-// common path).
-// s^2 (s/3 - L/2): int_0^s t (t - L) dt
-__device__ __forceinline__ float qcube(float s, float L) { return (s * s) * fmaf(s, 1.f / 3.f, -0.5f * L); }
-
-template <int NC, int NT, bool TRACK, bool FF, bool QUAD>
-__device__ __forceinline__ void multi_edges_lin(Cells<NC>& c, const Cold<NC, NT>& cold, int j, const float* G,
-                                                const float* D2, float L, float inv2L, const Consts& C, float& fn,
-                                                int k, int k_begin, int k_end)
-{
-    constexpr int NF = FF ? 3 : 6;                                  // carried field components
-    const float f = fn;
-    if (!(f >= 2.f * C.W)) return;
-    const float f0 = c.f[j];
-    const int b0 = c.bo[j] - row_base<NT>(j, C.n_bins);
-    const int m = (int)fminf(floorf(f * C.invW), 16777216.f);      // edges passed, >= 2
-    flush_acc<NC, FF>(C, c, j, b0, c.bo[j]);
-    // whole bins b0+i, i = 1..m-1, cover [i W, (i+1) W] from the start of bin b0
-    const int lo = max(1, -b0), hi = min(m - 1, C.n_bins - 1 - b0);
-    for (int i = lo; i <= hi; ++i) {
-        const float s0 = fmaf((float)i, C.W, -f0), s1 = s0 + C.W;
-        const float ramp = (s1 * s1 - s0 * s0) * inv2L;
-        float v[6];
-#pragma unroll
-        for (int q = 0; q < NF; ++q) v[q] = fmaf(c.gp[q][j], C.W - ramp, G[q] * ramp);
-        if (QUAD) {
-            const float cu = qcube(s1, L) - qcube(s0, L);
-#pragma unroll
-            for (int q = 0; q < NF; ++q) v[q] = fmaf(D2[q], cu, v[q]);
-        }
-        bin_b<NC, FF>(c, j, v, v + 3, v + 3);
-        flush(C, b0 + i, c.bo[j] + i, v[0], v[1], v[2], v[3], v[4], v[5]);
-    }
-    // bin b0+m holds [m W, f]
-    const float s0 = fmaf((float)m, C.W, -f0);
-    const float len = fmaf(-(float)m, C.W, f);
-    const float ramp = (L * L - s0 * s0) * inv2L;
-#pragma unroll
-    for (int q = 0; q < NF; ++q) c.acc[q][j] = fmaf(c.gp[q][j], len - ramp, G[q] * ramp);
-    if (QUAD) {
-        const float cu = qcube(L, L) - qcube(s0, L);
-#pragma unroll
-        for (int q = 0; q < NF; ++q) c.acc[q][j] = fmaf(D2[q], cu, c.acc[q][j]);
-    }
-    c.bo[j] += m;
-    fn = fminf(fmaxf(len, 0.f), C.W * 0.99999994f);
-    if (TRACK) {
-        if (b0 < 0 && b0 + m >= 0) cold.set(j, kBelow, k - k_begin + 1);
-        if (b0 < C.n_bins && b0 + m >= C.n_bins) cold.set(j, kAbove, k_end - k + 1);
-    }
-}
-
-// Walk modes.  kFast: the common step, with no code for an interval that passes two or more bin
-// edges; such an interval sets the cell's time to -inf, after which the cell crosses no edge and
-// flushes nothing for the rest of the tile.  kExact: the same arithmetic plus the multi-edge case;
-// used to walk a tile again (from its saved start) for a warp in which some cell stopped, flushing
-// only from the interval that stopped it onwards (earlier bins were flushed by the fast walk), and to
-// walk that warp's next tile at once.  Held field: exact_tile; step's kExact: interpolated fields.
-// Both walks evaluate every value with the same operations in the same order (no implicit
-// contraction), so they agree bit for bit up to that interval.
-enum { kFast = 0, kExact = 1 };
-
-// One interval for all cells of the thread: field of the sample (Eq. 1), the part of [f, f + du]
-// inside the current bin added to the running bin; a cell whose arrival time passes the bin edge
-// flushes the bin and starts the next one with the rest of the interval.  LAST: the interval ends
+// Fast step: one interval for all cells of the thread: field of the sample (Eq. 1), the part of
+// [f, f + du] inside the current bin added to the running bin; a cell whose arrival time passes the bin
+// edge flushes the bin and starts the next one with the rest of the interval.  LAST: the interval ends
 // on the exact FP64 anchors.  TRACK: bins may lie outside the window (checked, clipped intervals
-// counted).  ok: kExact only, false from the interval that stopped the fast walk onwards.
-template <int NC, int NT, int MODE, bool LAST, bool TRACK, bool FF, int LIN>
+// counted).
+template <int NC, int NT, bool LAST, bool TRACK, bool FF>
 __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& C, const Cold<NC, NT>& cold, int k,
-                                     int k_begin, int k_end, bool* ok, float ramp, bool again = false)
+                                     int k_begin, int k_end)
 {
-    constexpr int NF = FF ? 3 : 6;                  // carried field components (far field: E only)
-    constexpr bool QUAD = LIN == 2;                 // quadratic interpolation (RD_QUADRATIC)
     Field o[NC];
     float fn[NC];
-    float G[NC][6], L[NC], inv2L[NC], ramp1[NC];               // linear / quadratic interpolation only
-    float D2[NC][6], cu1[NC];                                  // quadratic interpolation only
-    // the trajectory's first two intervals have fewer than three fields behind them: no curvature
-    const float qon = (QUAD && k >= C.kq) ? 1.f : 0.f;
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
         if (FF)
@@ -330,138 +248,49 @@ __device__ __forceinline__ void step(Cells<NC>& c, const RecS& r, const Consts& 
         float t;
         if (LAST) {
             t = fmaf((float)(cold.bo_end(j) - c.bo[j]), C.W, cold.f_end(j));
-            if (MODE == kFast) t = c.f[j] == -INFINITY ? -INFINITY : t;
+            t = c.f[j] == -INFINITY ? -INFINITY : t;
         } else {
             t = fmaf(o[j].num, o[j].rden, c.f[j]);
         }
-        if (LIN) {
-            scaled_field(o[j], G[j]);
-            L[j] = t - c.f[j];
-            inv2L[j] = (0.5f * ramp) * fast_rcp(fmaxf(L[j], 1e-30f));
-            const float len1 = fminf(t, C.W) - c.f[j];
-            ramp1[j] = (len1 * len1) * inv2L[j];
-            // G0 (s1 - s0) + (G - G0) ramp = G0 (s1 - s0 - ramp) + G ramp
-            const float a1 = len1 - ramp1[j];
+        const float ws = (fminf(t, C.W) - c.f[j]) * o[j].S;
+        const float wb = ws * o[j].rinv;
 #pragma unroll
-            for (int i = 0; i < NF; ++i) c.acc[i][j] = fmaf(c.gp[i][j], a1, fmaf(G[j][i], ramp1[j], c.acc[i][j]));
-            if (QUAD) {
-                // D2 = ((G - G0) / L - (G0 - Gpp) / h) / (L + h), h the previous interval (ramp = 1 here,
-                // so 2 inv2L = 1/L); the part [0, len1] adds D2 int_0^len1 s (s - L) ds
-                const float iL = 2.f * inv2L[j];
-                const float ih = fast_rcp(c.hp[j]);
-                const float iLh = qon * fast_rcp(L[j] + c.hp[j]);
-                cu1[j] = qcube(len1, L[j]);
-#pragma unroll
-                for (int i = 0; i < NF; ++i) {
-                    D2[j][i] = fmaf(G[j][i] - c.gp[i][j], iL, -((c.gp[i][j] - c.gpp[i][j]) * ih)) * iLh;
-                    c.acc[i][j] = fmaf(D2[j][i], cu1[j], c.acc[i][j]);
-                }
-            }
-        } else {
-            const float ws = (fminf(t, C.W) - c.f[j]) * o[j].S;
-            const float wb = ws * o[j].rinv;
-#pragma unroll
-            for (int i = 0; i < 3; ++i) {
-                c.acc[i][j] = fmaf(o[j].E[i], ws, c.acc[i][j]);
-                if (!FF) c.acc[3 + i][j] = fmaf(o[j].B[i], wb, c.acc[3 + i][j]);
-            }
+        for (int i = 0; i < 3; ++i) {
+            c.acc[i][j] = fmaf(o[j].E[i], ws, c.acc[i][j]);
+            if (!FF) c.acc[3 + i][j] = fmaf(o[j].B[i], wb, c.acc[3 + i][j]);
         }
-        if (MODE == kFast)
-            t = t < 2.f * C.W ? t : -INFINITY;
-        else
-            ok[j] = ok[j] && (t < 2.f * C.W);
-        fn[j] = t;
-    }
-    if (MODE == kExact) {
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            multi_edges_lin<NC, NT, TRACK, FF, QUAD>(c, cold, j, G[j], D2[j], L[j], inv2L[j], C, fn[j], k, k_begin,
-                                                     k_end);
-        }
+        fn[j] = t < 2.f * C.W ? t : -INFINITY;
     }
 #pragma unroll
     for (int j = 0; j < NC; ++j) {
         // the arrival time passed the bin edge (a time exactly on the edge belongs to the upper bin)
         const bool cr = fn[j] >= C.W;
-        if (MODE == kFast && !TRACK) {
-            if (cr) {
-                float* a = bin_addr(C, c.bo[j]);
-                const float e[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
-                const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
-                float bb[3];
-                bin_b<NC, FF>(c, j, e, cb, bb);
-                if (!RD_CHECK || bin_ok(C, c.bo[j] - row_base<NT>(j, C.n_bins))) {
-                    red_add_v4(a, e[0], e[1], e[2], bb[0]);
-                    red_add_v2(a + 4, bb[1], bb[2]);
-                }
-                const float rem = fn[j] - C.W;
-                if (LIN) {
-                    const float ramp2 = fmaf(0.5f * ramp, L[j], -ramp1[j]);
-#pragma unroll
-                    for (int i = 0; i < NF; ++i) c.acc[i][j] = fmaf(c.gp[i][j], rem - ramp2, G[j][i] * ramp2);
-                    if (QUAD) {
-                        const float cu2 = qcube(L[j], L[j]) - cu1[j];       // the part [len1, L]
-#pragma unroll
-                        for (int i = 0; i < NF; ++i) c.acc[i][j] = fmaf(D2[j][i], cu2, c.acc[i][j]);
-                    }
-                } else {
-                    const float rs = rem * o[j].S;
-                    const float rbw = rs * o[j].rinv;
-#pragma unroll
-                    for (int i = 0; i < 3; ++i) {
-                        c.acc[i][j] = o[j].E[i] * rs;
-                        if (!FF) c.acc[3 + i][j] = o[j].B[i] * rbw;
-                    }
-                }
-                c.f[j] = rem;
-                c.bo[j] += 1;
-            } else {
-                c.f[j] = fn[j];
-            }
-        } else {
+        c.f[j] = fn[j];
+        if (cr) {
             const int b = TRACK || RD_CHECK ? c.bo[j] - row_base<NT>(j, C.n_bins) : 0;
-            const bool go = MODE == kFast || !(again && ok[j]);
-            const bool pr = cr && go && (TRACK ? (unsigned)b < (unsigned)C.n_bins : (!RD_CHECK || bin_ok(C, b)));
-            float* a = bin_addr(C, c.bo[j]);
             const float e[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
             const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
             float bb[3];
             bin_b<NC, FF>(c, j, e, cb, bb);
-            red_add_v4_if(pr, a, e[0], e[1], e[2], bb[0]);
-            red_add_v2_if(pr, a + 4, bb[1], bb[2]);
+            if (TRACK ? (unsigned)b < (unsigned)C.n_bins : (!RD_CHECK || bin_ok(C, b))) {
+                float* a = bin_addr(C, c.bo[j]);
+                red_add_v4(a, e[0], e[1], e[2], bb[0]);
+                red_add_v2(a + 4, bb[1], bb[2]);
+            }
             const float rem = fn[j] - C.W;
-            if (LIN) {
-                const float ramp2 = fmaf(0.5f * ramp, L[j], -ramp1[j]);
-                const float cu2 = QUAD ? qcube(L[j], L[j]) - cu1[j] : 0.f;
+            const float rs = rem * o[j].S;
+            const float rbw = rs * o[j].rinv;
 #pragma unroll
-                for (int i = 0; i < NF; ++i) {
-                    float v = fmaf(c.gp[i][j], rem - ramp2, G[j][i] * ramp2);
-                    if (QUAD) v = fmaf(D2[j][i], cu2, v);
-                    c.acc[i][j] = cr ? v : c.acc[i][j];
-                }
-            } else {
-                const float rs = rem * o[j].S;
-                const float rbw = rs * o[j].rinv;
-#pragma unroll
-                for (int i = 0; i < 3; ++i) {
-                    c.acc[i][j] = cr ? o[j].E[i] * rs : c.acc[i][j];
-                    if (!FF) c.acc[3 + i][j] = cr ? o[j].B[i] * rbw : c.acc[3 + i][j];
-                }
+            for (int i = 0; i < 3; ++i) {
+                c.acc[i][j] = o[j].E[i] * rs;
+                if (!FF) c.acc[3 + i][j] = o[j].B[i] * rbw;
             }
-            c.f[j] = cr ? rem : fn[j];
+            c.f[j] = rem;
+            c.bo[j] += 1;
             if (TRACK) {
-                if (cr && b == -1) cold.set(j, kBelow, k - k_begin + 1);
-                if (cr && b == C.n_bins - 1) cold.set(j, kAbove, k_end - k + 1);
+                if (b == -1) cold.set(j, kBelow, k - k_begin + 1);
+                if (b == C.n_bins - 1) cold.set(j, kAbove, k_end - k + 1);
             }
-            c.bo[j] += cr ? 1 : 0;
-        }
-        if (LIN) {
-#pragma unroll
-            for (int i = 0; i < NF; ++i) {
-                if (QUAD) c.gpp[i][j] = c.gp[i][j];
-                c.gp[i][j] = G[j][i];
-            }
-            if (QUAD) c.hp[j] = L[j];
         }
     }
 }
@@ -601,6 +430,11 @@ __device__ __forceinline__ void add_field(Cells<2>& c, const Field2& o, float2 w
 }
 
 __device__ __forceinline__ float half_of(float2 a, int j) { return j == 0 ? a.x : a.y; }
+__device__ __forceinline__ void set_half(float2& a, int j, float v)
+{
+    if (j == 0) a.x = v;
+    else a.y = v;
+}
 
 // Add the bin cell j is filling to global memory (the bin is inside the window).
 template <int NT, bool FF>
@@ -693,70 +527,304 @@ __device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, cons
     }
 }
 
-// Scratch of a warp in shared memory: save_cell words for each of its 32 NC cells.  The fast walk keeps
-// the state at the start of a tile there ([word][lane]: f, rpd, bo, below, above, acc[6], gp[6], and for
-// the quadratic interpolation gpp[6], hp); the exact walk, once it has taken that state back, hands its
-// runs of finished bins over there (add_runs: 16 words per lane).
-constexpr int save_cell(int lin) { return lin == 2 ? 24 : 17; }
+// ---------------------------------------------------------------------------------------------
+// Interpolated fields (two cells per thread as packed pairs).
+//
+// RD_LINEAR: over interval k (length L, arrival times f to f + L) the field goes linearly from F_{k-1} to
+// F_k, so the part [s0, s1] of the interval weighs F_{k-1} with (s1 - s0) - ramp and F_k with
+// ramp = (s1^2 - s0^2) / (2 L).  RD_HOLD_PREV is the same walk with the ramps scaled to zero.
+// RD_QUADRATIC adds D2 cu, D2 the second divided difference of F_{k-2}, F_{k-1}, F_k over their arrival
+// times (spacings h and L) and cu = int_{s0}^{s1} s (s - L) ds: weights cu alpha on F_k,
+// -cu (alpha + beta) on F_{k-1}, cu beta on F_{k-2}, alpha = 1 / (L (L + h)), beta = 1 / (h (L + h)).
+//
+// A sample's field so enters a bin with weights from two (three) intervals.  The walk does not add it once
+// per interval: it carries the weight that is still to come (Prev::r) and adds a field to the running bin
+// when its last interval is known, or when a bin ends in between.  That is one accumulation per interval
+// as for the held field, instead of two (three, and the differences that D2 is made of).  Measured on 200
+// electrons x 4000 steps x 16384 cells x 2048 bins: linear RD_LIN_MS, quadratic RD_QUAD_MS (a bin edge
+// passed in 18 % of the steps).
+// ---------------------------------------------------------------------------------------------
+struct Prev {                       // an earlier sample's field at both cells
+    float2 E[3], B[3], S, SB;       // E = S E', B = SB (d x E') (far-field limit: B unused)
+    float2 r;                       // weight of the running bin still to be added
+};
 
+struct LinState {
+    Prev p1, p2;                    // samples k-1 and (quadratic) k-2
+    float2 h;                       // quadratic: length of interval k-1
+};
 
-template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT>& cold, float* scratch)
+// int_0^s t (t - L) dt
+__device__ __forceinline__ float qcube(float s, float L) { return (s * s) * fmaf(s, 1.f / 3.f, -0.5f * L); }
+__device__ __forceinline__ float2 qcube2(float2 s, float2 L)
 {
-    float (*sv)[32] = reinterpret_cast<float (*)[32]>(scratch);
-    const int tid = threadIdx.x & 31;
-    constexpr int NF = FF ? 3 : 6;
-    constexpr int kSaveCell = save_cell(LIN);
+    return mul2(mul2(s, s), fma2(s, both(1.f / 3.f), mul2(both(-0.5f), L)));
+}
+
+template <bool FF>
+__device__ __forceinline__ void set_prev(Prev& p, const Field2& o, float2 r)
+{
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        sv[j * kSaveCell + 0][tid] = c.f[j];
-        sv[j * kSaveCell + 1][tid] = c.rpd[j];
-        sv[j * kSaveCell + 2][tid] = __int_as_float(c.bo[j]);
-        if (TRACK) {
-            sv[j * kSaveCell + 3][tid] = __int_as_float(cold.below(j));
-            sv[j * kSaveCell + 4][tid] = __int_as_float(cold.above(j));
-        }
+    for (int i = 0; i < 3; ++i) {
+        p.E[i] = o.E[i];
+        if (!FF) p.B[i] = o.B[i];
+    }
+    p.S = o.S;
+    if (!FF) p.SB = mul2(o.S, o.rinv);
+    p.r = r;
+}
+
+// running bin of cell j (+)= w times the sample's field
+template <bool FF, bool SET>
+__device__ __forceinline__ void add_prev(Cells<2>& c, const Prev& p, int j, float w)
+{
+    const float we = w * half_of(p.S, j), wb = FF ? 0.f : w * half_of(p.SB, j);
 #pragma unroll
-        for (int i = 0; i < NF; ++i) sv[j * kSaveCell + 5 + i][tid] = c.acc[i][j];
-        if (LIN) {
+    for (int i = 0; i < 3; ++i) {
+        c.acc[i][j] = SET ? half_of(p.E[i], j) * we : fmaf(half_of(p.E[i], j), we, c.acc[i][j]);
+        if (!FF) c.acc[3 + i][j] = SET ? half_of(p.B[i], j) * wb : fmaf(half_of(p.B[i], j), wb, c.acc[3 + i][j]);
+    }
+}
+
+template <bool FF>
+__device__ __forceinline__ void add_prev2(Cells<2>& c, const Prev& p, float2 w)
+{
+    const float2 we = mul2(w, p.S), wb = FF ? w : mul2(w, p.SB);
 #pragma unroll
-            for (int i = 0; i < NF; ++i) sv[j * kSaveCell + 11 + i][tid] = c.gp[i][j];
-        }
-        if (LIN == 2) {
-#pragma unroll
-            for (int i = 0; i < NF; ++i) sv[j * kSaveCell + 17 + i][tid] = c.gpp[i][j];
-            sv[j * kSaveCell + 23][tid] = c.hp[j];
+    for (int i = 0; i < 3; ++i) {
+        c.acc[i][0] = fmaf(p.E[i].x, we.x, c.acc[i][0]);
+        c.acc[i][1] = fmaf(p.E[i].y, we.y, c.acc[i][1]);
+        if (!FF) {
+            c.acc[3 + i][0] = fmaf(p.B[i].x, wb.x, c.acc[3 + i][0]);
+            c.acc[3 + i][1] = fmaf(p.B[i].y, wb.y, c.acc[3 + i][1]);
         }
     }
 }
 
-template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& cold, const float* scratch)
+// Fast step (unchecked window).  a: the sample whose field this interval completes (k-1; quadratic: k-2),
+// b: quadratic: sample k-1; a leaves as sample k (its place in the caller's rotation), b with its new r.
+// half_ramp: 1/2, or 0 to hold the previous field; curv: quadratic: 1, or 0 while fewer than three fields
+// lie behind.
+template <int NT, bool FF, bool QUAD>
+__device__ __forceinline__ void lin_step(Cells<2>& c, Prev& a, Prev& b, float2& h, const RecS& r, const Consts& C,
+                                         float half_ramp, float curv)
 {
-    const float (*sv)[32] = reinterpret_cast<const float (*)[32]>(scratch);
-    const int tid = threadIdx.x & 31;
-    constexpr int NF = FF ? 3 : 6;
-    constexpr int kSaveCell = save_cell(LIN);
+    Prev n;
+    float2 t, iL, al, be;
+    {
+        Field2 o;
+        field_pair<FF>(r, c, C, o);
+        t = fma2(o.num, o.rden, pair_of(c.f));
+        set_prev<FF>(n, o, both(0.f));
+    }
+    const float2 f = pair_of(c.f);
+    const float2 len1 = sub2(make_float2(fminf(t.x, C.W), fminf(t.y, C.W)), f), L = sub2(t, f);
+    iL = make_float2(fast_rcp(fmaxf(L.x, 1e-30f)), fast_rcp(fmaxf(L.y, 1e-30f)));
+    const float2 ramp1 = mul2(mul2(both(half_ramp), len1), mul2(len1, iL));
+    float2 wp, cu1;                 // weights of the first part: of sample k-1 (wp), of this sample (n.r)
+    if (QUAD) {
+        const float2 iLh = mul2(both(curv), rcp2(add2(L, h)));
+        al = mul2(iL, iLh);
+        be = mul2(rcp2(h), iLh);
+        cu1 = qcube2(len1, L);
+        add_prev2<FF>(c, a, fma2(cu1, be, a.r));
+        wp = add2(b.r, sub2(sub2(len1, ramp1), mul2(cu1, add2(al, be))));
+        n.r = fma2(cu1, al, ramp1);
+    } else {
+        add_prev2<FF>(c, a, add2(a.r, sub2(len1, ramp1)));
+        n.r = ramp1;
+    }
 #pragma unroll
-    for (int j = 0; j < NC; ++j) {
-        c.f[j] = sv[j * kSaveCell + 0][tid];
-        c.rpd[j] = sv[j * kSaveCell + 1][tid];
-        c.bo[j] = __float_as_int(sv[j * kSaveCell + 2][tid]);
+    for (int j = 0; j < 2; ++j) {
+        float fn = half_of(t, j);
+        fn = fn < 2.f * C.W ? fn : -INFINITY;
+        c.f[j] = fn;
+        if (fn >= C.W) {
+            if (QUAD) add_prev<FF, false>(c, b, j, half_of(wp, j));
+            add_prev<FF, false>(c, n, j, half_of(n.r, j));
+            red_bin<NT, FF>(C, c, j);
+            const float rem = fn - C.W, Lj = half_of(L, j);
+            const float ramp2 = fmaf(half_ramp, Lj, -half_of(ramp1, j));
+            if (QUAD) {
+                const float cu2 = qcube(Lj, Lj) - half_of(cu1, j);
+                add_prev<FF, true>(c, a, j, cu2 * half_of(be, j));
+                set_half(wp, j, rem - ramp2 - cu2 * (half_of(al, j) + half_of(be, j)));
+                set_half(n.r, j, fmaf(cu2, half_of(al, j), ramp2));
+            } else {
+                add_prev<FF, true>(c, a, j, rem - ramp2);
+                set_half(n.r, j, ramp2);
+            }
+            c.f[j] = rem;
+            c.bo[j] += 1;
+        }
+    }
+    a = n;
+    if (QUAD) {
+        b.r = wp;
+        h = L;
+    }
+}
+
+// Exact step: any number of edges, bins checked against the window, clipped intervals counted.  again: after
+// a fast walk that stopped; ok: false from the interval that stopped it onwards.
+template <int NT, bool FF, bool QUAD>
+__device__ __forceinline__ void lin_exact_step(Cells<2>& c, LinState& l, const RecS& r, const Consts& C,
+                                               const Cold<2, NT>& cold, bool last, int k, int k_begin, int k_end,
+                                               float half_ramp, bool again, bool* ok)
+{
+    Field2 o;
+    field_pair<FF>(r, c, C, o);
+    Prev n;
+    set_prev<FF>(n, o, both(0.f));
+    const float curv = (QUAD && k >= C.kq) ? 1.f : 0.f;
+    float2 rp = both(0.f), Lk;
+#pragma unroll
+    for (int j = 0; j < 2; ++j) {
+        const float f = c.f[j];
+        const float t = last ? fmaf((float)(cold.bo_end(j) - c.bo[j]), C.W, cold.f_end(j))
+                             : fmaf(half_of(o.num, j), half_of(o.rden, j), f);
+        const float L = t - f, iL = fast_rcp(fmaxf(L, 1e-30f));
+        const float iLh = QUAD ? curv * fast_rcp(L + half_of(l.h, j)) : 0.f;
+        const float al = QUAD ? iL * iLh : 0.f, be = QUAD ? fast_rcp(half_of(l.h, j)) * iLh : 0.f;
+        // weights of the part [s0, s0 + len] of the interval: of samples k-2, k-1 and k
+        auto weights = [&](float s0, float len, float& w2, float& w1, float& w0) {
+            const float s1 = s0 + len;
+            const float ramp = (half_ramp * iL) * (len * (s0 + s1));
+            const float cu = QUAD ? qcube(s1, L) - qcube(s0, L) : 0.f;
+            w2 = cu * be;
+            w1 = (len - ramp) - cu * (al + be);
+            w0 = fmaf(cu, al, ramp);
+        };
+        ok[j] = ok[j] && t < 2.f * C.W;
+        const bool go = !(again && ok[j]);
+        int m = t >= C.W ? 1 : 0;
+        float rem = t - C.W;
+        if (t >= 2.f * C.W) {
+            m = max(2, (int)fminf(floorf(t * C.invW), 16777216.f));
+            rem = fminf(fmaxf(fmaf(-(float)m, C.W, t), 0.f), C.W * 0.99999994f);
+        }
+        float w2, w1, w0;
+        weights(0.f, fminf(t, C.W) - f, w2, w1, w0);
+        if (QUAD) {
+            add_prev<FF, false>(c, l.p2, j, half_of(l.p2.r, j) + w2);
+            w1 += half_of(l.p1.r, j);
+        } else {
+            add_prev<FF, false>(c, l.p1, j, half_of(l.p1.r, j) + w1);
+        }
+        if (m > 0) {
+            const int b0 = c.bo[j] - row_base<NT>(j, C.n_bins);
+            if (QUAD) add_prev<FF, false>(c, l.p1, j, w1);
+            add_prev<FF, false>(c, n, j, w0);
+            if (go) flush_acc<2, FF>(C, c, j, b0, c.bo[j]);
+            // whole bins b0 + i
+            const int hi = go ? min(m - 1, C.n_bins - 1 - b0) : 0;
+            for (int i = max(1, -b0); i <= hi; ++i) {
+                weights(fmaf((float)i, C.W, -f), C.W, w2, w1, w0);
+                add_prev<FF, true>(c, n, j, w0);
+                add_prev<FF, false>(c, l.p1, j, w1);
+                if (QUAD) add_prev<FF, false>(c, l.p2, j, w2);
+                flush_acc<2, FF>(C, c, j, b0 + i, c.bo[j] + i);
+            }
+            weights(fmaf((float)m, C.W, -f), rem, w2, w1, w0);
+            add_prev<FF, true>(c, QUAD ? l.p2 : l.p1, j, QUAD ? w2 : w1);
+            c.bo[j] += m;
+            if (b0 < 0 && b0 + m >= 0) cold.set(j, kBelow, k - k_begin + 1);
+            if (b0 < C.n_bins && b0 + m >= C.n_bins) cold.set(j, kAbove, k_end - k + 1);
+        }
+        c.f[j] = m > 0 ? rem : t;
+        set_half(n.r, j, w0);
+        set_half(rp, j, w1);
+        set_half(Lk, j, L);
+    }
+    if (QUAD) {
+        l.p2 = l.p1;
+        l.p2.r = rp;
+        l.h = Lk;
+    }
+    l.p1 = n;
+}
+
+// The weights still to come of the earlier samples' fields, into the running bin (at the chunk's end).
+template <bool FF, bool QUAD>
+__device__ __forceinline__ void settle(Cells<2>& c, const LinState& l)
+{
+    add_prev2<FF>(c, l.p1, l.p1.r);
+    if (QUAD) add_prev2<FF>(c, l.p2, l.p2.r);
+}
+
+// Scratch of a warp in shared memory: save_cell words for each of its 32 NC cells.  The fast walk keeps
+// the state at the start of a tile there ([word][lane]: f, rpd, bo, below, above, acc[6]; interpolated
+// fields: p1, and for the quadratic interpolation p2 and h); the exact walk, once it has taken that state
+// back, hands its runs of finished bins over there (add_runs: 16 words per lane).
+constexpr int save_cell(int lin) { return lin == 2 ? 30 : lin == 1 ? 20 : 17; }
+
+template <int NC, int NT, bool TRACK, bool FF>
+__device__ __forceinline__ void save_state(const Cells<NC>& c, const Cold<NC, NT>& cold, float (*sv)[32], int words)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < NC; ++j, sv += words) {
+        sv[0][lane] = c.f[j];
+        sv[1][lane] = c.rpd[j];
+        sv[2][lane] = __int_as_float(c.bo[j]);
         if (TRACK) {
-            cold.set(j, kBelow, sv[j * kSaveCell + 3][tid]);
-            cold.set(j, kAbove, sv[j * kSaveCell + 4][tid]);
+            sv[3][lane] = __int_as_float(cold.below(j));
+            sv[4][lane] = __int_as_float(cold.above(j));
         }
 #pragma unroll
-        for (int i = 0; i < NF; ++i) c.acc[i][j] = sv[j * kSaveCell + 5 + i][tid];
-        if (LIN) {
+        for (int i = 0; i < (FF ? 3 : 6); ++i) sv[5 + i][lane] = c.acc[i][j];
+    }
+}
+
+template <int NC, int NT, bool TRACK, bool FF>
+__device__ __forceinline__ void restore_state(Cells<NC>& c, const Cold<NC, NT>& cold, const float (*sv)[32], int words)
+{
+    const int lane = threadIdx.x & 31;
 #pragma unroll
-            for (int i = 0; i < NF; ++i) c.gp[i][j] = sv[j * kSaveCell + 11 + i][tid];
+    for (int j = 0; j < NC; ++j, sv += words) {
+        c.f[j] = sv[0][lane];
+        c.rpd[j] = sv[1][lane];
+        c.bo[j] = __float_as_int(sv[2][lane]);
+        if (TRACK) {
+            cold.set(j, kBelow, sv[3][lane]);
+            cold.set(j, kAbove, sv[4][lane]);
         }
-        if (LIN == 2) {
 #pragma unroll
-            for (int i = 0; i < NF; ++i) c.gpp[i][j] = sv[j * kSaveCell + 17 + i][tid];
-            c.hp[j] = sv[j * kSaveCell + 23][tid];
+        for (int i = 0; i < (FF ? 3 : 6); ++i) c.acc[i][j] = sv[5 + i][lane];
+    }
+}
+
+template <bool FF>
+__device__ __forceinline__ void save_prev(const Prev& p, float (*sv)[32], int words)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 2; ++j, sv += words) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            sv[i][lane] = half_of(p.E[i], j);
+            if (!FF) sv[3 + i][lane] = half_of(p.B[i], j);
         }
+        sv[6][lane] = half_of(p.S, j);
+        if (!FF) sv[7][lane] = half_of(p.SB, j);
+        sv[8][lane] = half_of(p.r, j);
+    }
+}
+
+template <bool FF>
+__device__ __forceinline__ void restore_prev(Prev& p, const float (*sv)[32], int words)
+{
+    const int lane = threadIdx.x & 31;
+#pragma unroll
+    for (int j = 0; j < 2; ++j, sv += words) {
+#pragma unroll
+        for (int i = 0; i < 3; ++i) {
+            set_half(p.E[i], j, sv[i][lane]);
+            if (!FF) set_half(p.B[i], j, sv[3 + i][lane]);
+        }
+        set_half(p.S, j, sv[6][lane]);
+        if (!FF) set_half(p.SB, j, sv[7][lane]);
+        set_half(p.r, j, sv[8][lane]);
     }
 }
 
@@ -910,59 +978,98 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
 }
 
 // The fast walk of one tile; false if it met an interval of two or more edges (the state is then back at the
-// tile's start).
+// tile's start).  Interpolated fields: only in windows that hold every arrival (no TRACK).
 template <int NC, int NT, bool TRACK, bool FF, int LIN>
-__device__ __forceinline__ bool fast_tile(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
-                                          float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
-                                          float* scratch)
+__device__ __forceinline__ bool fast_tile(Cells<NC>& c, LinState& l, const RecS* tile, int cnt, bool last_tile,
+                                          const Consts& C, float half_ramp, const Cold<NC, NT>& cold, int k0, int k_begin,
+                                          int k_end, float* scratch)
 {
+    constexpr bool QUAD = LIN == 2;
+    constexpr int words = save_cell(LIN);
+    float (*sv)[32] = reinterpret_cast<float (*)[32]>(scratch);
     const int n_regular = last_tile ? cnt - 1 : cnt;
-    bool ok[NC];
-    save_state<NC, NT, TRACK, FF, LIN>(c, cold, scratch);
-    if constexpr (NC == 2 && !TRACK && LIN == 0) {
+    save_state<NC, NT, TRACK, FF>(c, cold, sv, words);
+    if constexpr (LIN != 0) {
+        save_prev<FF>(l.p1, sv + 11, words);
+        if (QUAD) {
+            const int lane = threadIdx.x & 31;
+            save_prev<FF>(l.p2, sv + 20, words);
+            sv[29][lane] = l.h.x;
+            sv[words + 29][lane] = l.h.y;
+        }
+        int i = 0;
+        if constexpr (QUAD) {
+            auto curv = [&](int q) { return k0 + q >= C.kq ? 1.f : 0.f; };
+#pragma unroll 1
+            for (; i + 1 < n_regular; i += 2) {
+                lin_step<NT, FF, true>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i));
+                lin_step<NT, FF, true>(c, l.p1, l.p2, l.h, tile[i + 1], C, half_ramp, curv(i + 1));
+            }
+            if (i < n_regular) {
+                lin_step<NT, FF, true>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i));
+                const Prev x = l.p1;
+                l.p1 = l.p2;
+                l.p2 = x;
+            }
+        } else {
+            // (two per iteration, so that sample k's field stays where it was formed)
+#pragma unroll 2
+            for (; i < n_regular; ++i) lin_step<NT, FF, false>(c, l.p1, l.p2, l.h, tile[i], C, half_ramp, 0.f);
+        }
+    } else if constexpr (NC == 2 && !TRACK) {
         int i = 0;
 #pragma unroll 1
         for (; i + 1 < n_regular; i += 2) two_steps_pair<NT, FF>(c, tile[i], tile[i + 1], C);
-        if (i < n_regular)
-            step<NC, NT, kFast, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
+        if (i < n_regular) step<NC, NT, false, TRACK, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
     } else {
 #pragma unroll kUnroll
-        for (int i = 0; i < n_regular; ++i)
-            step<NC, NT, kFast, false, TRACK, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp);
+        for (int i = 0; i < n_regular; ++i) step<NC, NT, false, TRACK, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
     }
-    if (last_tile)
-        step<NC, NT, kFast, true, TRACK, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp);
+    if constexpr (LIN == 0) {
+        if (last_tile) step<NC, NT, true, TRACK, FF>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end);
+    }
     bool stopped = false;
 #pragma unroll
     for (int j = 0; j < NC; ++j) stopped = stopped || c.f[j] == -INFINITY;
-    if (!__any_sync(0xffffffffu, stopped)) return true;
-    restore_state<NC, NT, TRACK, FF, LIN>(c, cold, scratch);
+    if (!__any_sync(0xffffffffu, stopped)) {
+        if constexpr (LIN != 0) {
+            bool ok[2] = {true, true};
+            if (last_tile)
+                lin_exact_step<NT, FF, QUAD>(c, l, tile[cnt - 1], C, cold, true, k_end, k_begin, k_end, half_ramp, false,
+                                             ok);
+        }
+        return true;
+    }
+    restore_state<NC, NT, TRACK, FF>(c, cold, sv, words);
+    if constexpr (LIN != 0) {
+        restore_prev<FF>(l.p1, sv + 11, words);
+        if (QUAD) {
+            const int lane = threadIdx.x & 31;
+            restore_prev<FF>(l.p2, sv + 20, words);
+            l.h = make_float2(sv[29][lane], sv[words + 29][lane]);
+        }
+    }
     return false;
 }
 
 // The exact walk of one tile; again: after a fast walk that stopped (earlier bins are flushed).  Returns
 // whether the warp met an interval of two or more edges.
 template <int NC, int NT, bool FF, int LIN>
-__device__ __forceinline__ bool exact_walk(Cells<NC>& c, const RecS* tile, int cnt, bool last_tile, const Consts& C,
-                                           float ramp, const Cold<NC, NT>& cold, int k0, int k_begin, int k_end,
-                                           float* scratch, bool again, bool track)
+__device__ __forceinline__ bool exact_walk(Cells<NC>& c, LinState& l, const RecS* tile, int cnt, bool last_tile,
+                                           const Consts& C, float half_ramp, const Cold<NC, NT>& cold, int k0, int k_begin,
+                                           int k_end, float* scratch, bool again, bool track)
 {
     if constexpr (LIN == 0) {
         return exact_tile<NC, NT, FF>(c, tile, cnt, last_tile, C, cold, k0, k_begin, k_end, scratch, again, track);
     } else {
-        const int n_regular = last_tile ? cnt - 1 : cnt;
-        bool ok[NC];
-#pragma unroll
-        for (int j = 0; j < NC; ++j) ok[j] = true;
+        bool ok[2] = {true, true};
 #pragma unroll 1
-        for (int i = 0; i < n_regular; ++i)
-            step<NC, NT, kExact, false, true, FF, LIN>(c, tile[i], C, cold, k0 + i, k_begin, k_end, ok, ramp, again);
-        if (last_tile)
-            step<NC, NT, kExact, true, true, FF, LIN>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end, ok, ramp, again);
-        bool met = false;
-#pragma unroll
-        for (int j = 0; j < NC; ++j) met = met || !ok[j];
-        return __any_sync(0xffffffffu, met);
+        for (int i = 0; i < cnt; ++i) {
+            const bool last = last_tile && i == cnt - 1;        // (not walked by a fast walk that stopped)
+            lin_exact_step<NT, FF, LIN == 2>(c, l, tile[i], C, cold, last, k0 + i, k_begin, k_end, half_ramp,
+                                             again && !last, ok);
+        }
+        return __any_sync(0xffffffffu, !ok[0] || !ok[1]);
     }
 }
 
@@ -1032,6 +1139,7 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         c.py[j] = c.pz[j] = 0.f;
         c.nlx[j] = c.nly[j] = c.nlz[j] = 0.f;
         int bo_end = rb, below = -1;
+        hp0[j] = 1.f;
         float f_end = 0.f;
 #pragma unroll
         for (int i = 0; i < 6; ++i) c.acc[i][j] = 0.f;
@@ -1049,7 +1157,6 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
                 ue = arrival_bins(xe[0], xe[1], xe[2], cl, P.t0, k_end, P.dt, P.inv_dt_det, Re);
             }
             const bool live = (ue > 0.0) && (ua < (double)P.n_bins);
-            hp0[j] = 1.f;
             if (q_prev && live) {
                 const double* xq = xp + 3 * (size_t)(k_begin - 2);
                 double Rq;
@@ -1099,41 +1206,24 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) crossed += __shfl_xor_sync(0xffffffffu, crossed, o);
     if ((tid & 31) == 0 && crossed) atomicAdd(&P.counters->crossings, crossed);
-    // clip tracking costs instructions in the bin-crossing path: only CTAs that need it use it
-    if (LIN) {
+    LinState l;
+    if constexpr (LIN != 0) {
         // field of the sample before the chunk; a trajectory's first interval holds F_1 (sample 0
         // has no field), so the first chunk starts from the field of sample 1 itself
-        const RecS r0 = rec[k_begin > 1 ? k_begin - 1 : 1];
-#pragma unroll
-        for (int j = 0; j < NC; ++j) {
-            Field o;
-            float rtmp = c.rpd[j];
-            if (FF)
-                field_at_ff(r0, c.px[j], c.py[j], c.pz[j], c.rpd[j], c.nlx[j], c.nly[j], c.nlz[j], o);
-            else
-                field_at(r0, c.px[j], c.py[j], c.pz[j], rtmp, C, o);
-            float G[6];
-            scaled_field(o, G);
-#pragma unroll
-            for (int i = 0; i < 6; ++i) c.gp[i][j] = G[i];      // far field: only E is read
-            if (QUAD) {
-                // the field two samples before the chunk and the interval before it (used from the
-                // trajectory's third interval on)
-                c.hp[j] = hp0[j];
-                if (q_prev) {
-                    const RecS r1 = rec[k_begin - 2];
-                    float rtmp1 = c.rpd[j];
-                    if (FF)
-                        field_at_ff(r1, c.px[j], c.py[j], c.pz[j], c.rpd[j], c.nlx[j], c.nly[j], c.nlz[j], o);
-                    else
-                        field_at(r1, c.px[j], c.py[j], c.pz[j], rtmp1, C, o);
-                    scaled_field(o, G);
-                }
-#pragma unroll
-                for (int i = 0; i < 6; ++i) c.gpp[i][j] = G[i];
-            }
+        const float rpd[2] = {c.rpd[0], c.rpd[1]};
+        Field2 o;
+        field_pair<FF>(rec[k_begin > 1 ? k_begin - 1 : 1], c, C, o);
+        set_prev<FF>(l.p1, o, both(0.f));
+        if (QUAD) {
+            // the field two samples before the chunk and the interval before it (used from the
+            // trajectory's third interval on)
+            l.h = make_float2(hp0[0], hp0[1]);
+            if (q_prev) field_pair<FF>(rec[k_begin - 2], c, C, o);
+            set_prev<FF>(l.p2, o, both(0.f));
         }
+        set_pair(c.rpd, pair_of(rpd));
     }
+    // clip tracking costs instructions in the bin-crossing path: only CTAs that need it use it
     const bool track = __syncthreads_or(partial) != 0;
     many = __any_sync(0xffffffffu, many);
 
@@ -1156,16 +1246,23 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         const bool last_tile = (t == n_tiles - 1);
         // many (warp-uniform): the warp's last tile met intervals of two or more edges (at the start: the
         // anchors say more than one edge an interval), so this one goes to the exact walk at once
-        const float ramp = P.lin == 2 ? 0.f : 1.f;
+        const float half_ramp = P.lin == 2 ? 0.f : 0.5f;
         bool done = false;
-        if (!many)
-            done = track ? fast_tile<NC, NT, true, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin,
-                                                            k_end, scratch)
-                         : fast_tile<NC, NT, false, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin,
-                                                             k_end, scratch);
+        if constexpr (LIN == 0) {
+            if (!many)
+                done = track ? fast_tile<NC, NT, true, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
+                                                                k_begin, k_end, scratch)
+                             : fast_tile<NC, NT, false, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
+                                                                 k_begin, k_end, scratch);
+        } else {
+            many = many || track;
+            if (!many)
+                done = fast_tile<NC, NT, false, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin,
+                                                         k_end, scratch);
+        }
         if (!done)
-            many = exact_walk<NC, NT, FF, LIN>(c, tile[buf], cnt, last_tile, C, ramp, cold, k0, k_begin, k_end, scratch,
-                                               !many, track);
+            many = exact_walk<NC, NT, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin, k_end,
+                                               scratch, !many, track);
         __syncthreads();
         if (tid == 0 && t + 2 < n_tiles) {
             fence_proxy_async();
@@ -1176,6 +1273,7 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
         }
     }
     g_base += (unsigned)n_tiles;
+    if constexpr (LIN != 0) settle<FF, QUAD>(c, l);
     // close the last bin; count clipped intervals
     unsigned long long clipped = 0;
 #pragma unroll
