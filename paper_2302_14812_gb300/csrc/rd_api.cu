@@ -57,8 +57,10 @@ struct rd_detector {
     int spec_n = 0;
     std::vector<float2> spec_tw_host;
     // streamed deposits: the last sample (x, u) of every particle from the previous call
-    void* strm_last = nullptr;       // x then u, each [n_part][3][3] doubles (last samples)
+    void* strm_last = nullptr;       // two buffers (the current one: strm_cur) of x then u, each [n_part][3][3]
+                                     // doubles: the last samples
     size_t strm_last_bytes = 0;
+    int strm_cur = 0;
     void* strm_stage = nullptr;      // this call's samples with the stored one in front, and q
     size_t strm_stage_bytes = 0;
     int strm_n_part = -1;            // -1: no stream in progress
@@ -1256,28 +1258,35 @@ rd_status rd_deposit_stream(rd_detector* d, const rd_traj* t, rd_stream stream)
     const size_t row = one * (size_t)ns, mrow = one * (size_t)m;
     st = ensure(&d->strm_stage, &d->strm_stage_bytes, 2 * row * np + sizeof(double) * np, s, "stream staging");
     if (st != RD_OK) return st;
+    const size_t state = 2 * one * 3 * (size_t)np;          // bytes of one state buffer
     if (!cont) {
-        st = ensure(&d->strm_last, &d->strm_last_bytes, 2 * one * 3 * np, s, "stream state");
+        st = ensure(&d->strm_last, &d->strm_last_bytes, 2 * state, s, "stream state");
         if (st != RD_OK) return st;
     }
     double* xs = static_cast<double*>(d->strm_stage);
     double* us = xs + (size_t)np * ns * 3;
     double* qs = us + (size_t)np * ns * 3;
-    double* lx = static_cast<double*>(d->strm_last);        // [np][have][3], have <= 3
-    double* lu = lx + (size_t)np * 3 * 3;
-    const cudaMemcpyKind kind = t->mem == RD_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
-    RD_CUDA(cudaMemcpy2DAsync(xs + 3 * have, row, t->x, mrow, mrow, np, kind, s), "stream x");
-    RD_CUDA(cudaMemcpy2DAsync(us + 3 * have, row, t->u, mrow, mrow, np, kind, s), "stream u");
-    if (have > 0) {
-        RD_CUDA(cudaMemcpy2DAsync(xs, row, lx, one * have, one * have, np, cudaMemcpyDeviceToDevice, s), "stream x");
-        RD_CUDA(cudaMemcpy2DAsync(us, row, lu, one * have, one * have, np, cudaMemcpyDeviceToDevice, s), "stream u");
+    const double* lx = reinterpret_cast<double*>(static_cast<char*>(d->strm_last) + state * d->strm_cur);
+    double* nx = reinterpret_cast<double*>(static_cast<char*>(d->strm_last) + state * (1 - d->strm_cur));
+    const size_t lu = (size_t)np * 3 * 3;                   // u behind x in a state buffer
+    const int kept = std::min(keep, ns);
+    // the kept samples and the new ones, and the state of the next call (in the other buffer, which
+    // becomes current once this call has gone through)
+    const double *tx = t->x, *tu = t->u;
+    const double* tq = t->q;
+    if (t->mem == RD_MEM_HOST) {
+        RD_CUDA(cudaMemcpy2DAsync(xs + 3 * have, row, t->x, mrow, mrow, np, cudaMemcpyHostToDevice, s), "stream x");
+        RD_CUDA(cudaMemcpy2DAsync(us + 3 * have, row, t->u, mrow, mrow, np, cudaMemcpyHostToDevice, s), "stream u");
+        if (t->q) RD_CUDA(cudaMemcpyAsync(qs, t->q, sizeof(double) * np, cudaMemcpyHostToDevice, s), "stream q");
+        tx = tu = nullptr;                                  // already in place
+        tq = t->q ? qs : nullptr;
     }
-    if (t->q) RD_CUDA(cudaMemcpyAsync(qs, t->q, sizeof(double) * np, kind, s), "stream q");
+    RD_CUDA(launch_stream_gather(np, m, have, kept, lx, lx + lu, tx, tu, xs, us, nx, nx + lu, s), "stream samples");
     rd_traj staged = *t;
     staged.n_samples = ns;
     staged.x = xs;
     staged.u = us;
-    staged.q = t->q ? qs : nullptr;
+    staged.q = tq;
     staged.mem = RD_MEM_DEVICE;
     staged.t0 = t->t0 - have * t->dt;
     // intervals already deposited by earlier calls are not deposited again; the staged sample 0 is
@@ -1285,13 +1294,7 @@ rd_status rd_deposit_stream(rd_detector* d, const rd_traj* t, rd_stream stream)
     const long long count0 = cont ? d->strm_count : 0;
     st = deposit_from(d, &staged, stream, std::max(1, have), (int)std::min<long long>(count0 - have, 1 << 30));
     if (st != RD_OK) return st;
-    const int kept = std::min(keep, ns);
-    RD_CUDA(cudaMemcpy2DAsync(lx, one * kept, xs + 3 * (size_t)(ns - kept), row, one * kept, np,
-                              cudaMemcpyDeviceToDevice, s),
-            "stream state");
-    RD_CUDA(cudaMemcpy2DAsync(lu, one * kept, us + 3 * (size_t)(ns - kept), row, one * kept, np,
-                              cudaMemcpyDeviceToDevice, s),
-            "stream state");
+    d->strm_cur = 1 - d->strm_cur;
     d->strm_n_part = np;
     d->strm_have = kept;
     d->strm_count = count0 + m;

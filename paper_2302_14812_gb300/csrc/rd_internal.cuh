@@ -278,6 +278,12 @@ cudaError_t launch_gbeta_to_gu(const double* u, const double* gbeta, double* gu,
 // run-time coupling (rd_push.cu): Boris steps in a uniform magnetic field B[3] (host array)
 cudaError_t launch_push_boris(int n_part, int n_steps, double dt, const double* B, double qm, double* x, double* u,
                               double* x_out, double* u_out, cudaStream_t s);
+// streamed deposits (rd_push.cu): [n_part][have + m][3] samples xs, us = the `have` kept ones (lx, lu:
+// [n_part][have][3]) then the m new ones (x, u: [n_part][m][3]; null: already in place), and the last `kept`
+// of them as the next call's state (nx, nu: [n_part][kept][3], another buffer than lx, lu)
+cudaError_t launch_stream_gather(int n_part, int m, int have, int kept, const double* lx, const double* lu,
+                                 const double* x, const double* u, double* xs, double* us, double* nx, double* nu,
+                                 cudaStream_t s);
 // diagnostics (rd_diag.cu): FMA throughput of the current device in TFLOP/s (one FMA = 2 flops), and one
 // CTA whose bounded wait on an mbarrier phase that nothing completes runs out after limit_ns (the
 // expiry is recorded in *errors as the kernels record it)

@@ -53,7 +53,52 @@ __global__ void k_push_boris(int n_part, int n_steps, double dt, double bx, doub
     u[3 * p + 2] = U[2];
 }
 
+// One thread per value (particle, staged sample, component) of x and u.  A streamed call is a few
+// microseconds of copying: one launch instead of seven strided copies (256 particles x 25 samples: 12 us and
+// seven enqueues a call, 3 us and one).
+__global__ void k_stream_gather(long long total, int m3, int have3, int kept3, const double* __restrict__ lx,
+                                const double* __restrict__ lu, const double* __restrict__ x,
+                                const double* __restrict__ u, double* xs, double* us, double* __restrict__ nx,
+                                double* __restrict__ nu)
+{
+    const int row = m3 + have3;
+    for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
+         e += (long long)gridDim.x * blockDim.x) {
+        const long long p = e <= 0x7fffffffLL ? (int)e / row : e / row;
+        const int r = (int)(e - p * row);
+        double vx, vu;
+        if (r < have3) {
+            vx = lx[p * have3 + r];
+            vu = lu[p * have3 + r];
+        } else if (x) {
+            vx = x[p * m3 + (r - have3)];
+            vu = u[p * m3 + (r - have3)];
+        } else {
+            vx = xs[e];
+            vu = us[e];
+        }
+        if (r < have3 || x) {
+            xs[e] = vx;
+            us[e] = vu;
+        }
+        if (r >= row - kept3) {
+            nx[p * kept3 + (r - (row - kept3))] = vx;
+            nu[p * kept3 + (r - (row - kept3))] = vu;
+        }
+    }
+}
+
 }  // namespace
+
+cudaError_t launch_stream_gather(int n_part, int m, int have, int kept, const double* lx, const double* lu,
+                                 const double* x, const double* u, double* xs, double* us, double* nx, double* nu,
+                                 cudaStream_t s)
+{
+    const long long total = 3LL * n_part * (m + have);
+    k_stream_gather<<<grid_stride_blocks(total, 256, 8), 256, 0, s>>>(total, 3 * m, 3 * have, 3 * kept, lx, lu, x, u, xs,
+                                                                      us, nx, nu);
+    return cudaGetLastError();
+}
 
 cudaError_t launch_push_boris(int n_part, int n_steps, double dt, const double* B, double qm, double* x, double* u,
                               double* x_out, double* u_out, cudaStream_t s)
