@@ -77,6 +77,19 @@ class rd_stats(ctypes.Structure):
 
 _lock = threading.Lock()
 _lib = None
+_torch_mod = None       # torch once imported, False if there is none
+
+
+def _torch():
+    """torch, or None where it is not installed."""
+    global _torch_mod
+    if _torch_mod is None:
+        try:
+            import torch
+            _torch_mod = torch
+        except ImportError:
+            _torch_mod = False
+    return _torch_mod or None
 
 
 def library_path() -> str:
@@ -87,6 +100,8 @@ def library_path() -> str:
 def load_library(build_if_missing: bool = True):
     """Load librd.so (building it first if it is missing and nvcc is available)."""
     global _lib
+    if _lib is not None:                # set once, under the lock, when the library is complete
+        return _lib
     with _lock:
         if _lib is not None:
             return _lib
@@ -142,14 +157,16 @@ def _check(status: int, where: str):
         raise RDError(status, where, load_library().rd_last_error().decode(errors="replace"))
 
 
+# A call on a small detector is a few microseconds of GPU work, so its arguments are marshalled without
+# creating stream, device or tensor objects on the way (one electron on 64 cells, zero + deposit + read:
+# 55 us of host time a pass with them, 30 us without).
 def _stream_ptr(stream) -> Optional[int]:
     if stream is None:
-        try:
-            import torch
-            if torch.cuda.is_available():
-                return torch.cuda.current_stream().cuda_stream
-        except ImportError:
-            pass
+        t = _torch()
+        if t is not None and t.cuda.is_available():
+            if not t.cuda.is_initialized():
+                t.cuda.init()
+            return t._C._cuda_getCurrentRawStream(t._C._cuda_getDevice())     # current_stream().cuda_stream
         return None
     if isinstance(stream, int):
         return stream
@@ -329,16 +346,13 @@ def rd_version() -> str:
 # --------------------------------------------------------------------------------------------
 def _as_f64(a, keep):
     """(pointer, mem, n_elements) of an FP64 C-contiguous view of a torch tensor or array."""
-    try:
-        import torch
-        if isinstance(a, torch.Tensor):
-            t = a.detach()
-            if t.dtype != torch.float64 or not t.is_contiguous():
-                t = t.to(torch.float64).contiguous()
-            keep.append(t)
-            return t.data_ptr(), (RD_MEM_DEVICE if t.is_cuda else RD_MEM_HOST), t.numel()
-    except ImportError:
-        pass
+    torch = _torch()
+    if torch is not None and isinstance(a, torch.Tensor):
+        t = a.detach() if a.requires_grad else a
+        if t.dtype is not torch.float64 or not t.is_contiguous():
+            t = t.to(torch.float64).contiguous()
+        keep.append(t)
+        return t.data_ptr(), (RD_MEM_DEVICE if t.is_cuda else RD_MEM_HOST), t.numel()
     arr = np.ascontiguousarray(np.asarray(a, dtype=np.float64))
     keep.append(arr)
     return arr.ctypes.data, RD_MEM_HOST, arr.size
@@ -421,7 +435,7 @@ class RadiationDetector:
             B = np.empty_like(E)
             rd_read_fields(self._h, E.ctypes.data, B.ctypes.data, code, RD_MEM_HOST, stream)
             return E, B
-        import torch
+        torch = _torch()
         tdt = torch.float32 if code == RD_F32 else torch.float64
         E = torch.empty((self.n_pix, self.n_bins, 3), dtype=tdt, device=device)
         B = torch.empty_like(E)

@@ -4,6 +4,7 @@
 #include <cuda_runtime.h>
 #include <math.h>
 #include <stdarg.h>
+#include <stddef.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -29,7 +30,7 @@ struct rd_detector {
     D4* cells = nullptr;             // [n_pix]
     void* fields = nullptr;          // internal accumulators
     size_t field_bytes = 0;
-    DevCounters* counters = nullptr;
+    DevCounters* counters = nullptr; // in the fields' allocation, right behind them (counters_at)
     DevCounters* host_counters = nullptr;   // page-locked copy target of `counters`
     void* rec = nullptr;             // per-sample records
     size_t rec_bytes = 0;
@@ -83,6 +84,9 @@ struct rd_detector {
 };
 
 namespace {
+
+// The counters follow the fields in one allocation, so that one memset clears both.
+size_t counters_at(size_t field_bytes) { return (field_bytes + 15) & ~size_t(15); }
 
 thread_local std::string g_err;
 unsigned long long g_next_id = 1;   // detector ids (host side, monotonic)
@@ -414,19 +418,18 @@ rd_status rd_create_detector(const rd_detector_desc* desc, rd_stream stream, rd_
     d->dt_det = desc->dt_det;
     d->field_bytes = (size_t)desc->n_pix * desc->n_bins * per_bin;
     cudaError_t e = cudaMalloc(&d->cells, sizeof(D4) * cells.size());
-    if (e == cudaSuccess) e = cudaMalloc(&d->fields, d->field_bytes);
-    if (e == cudaSuccess) e = cudaMalloc(&d->counters, sizeof(DevCounters));
+    const size_t at = counters_at(d->field_bytes);
+    if (e == cudaSuccess) e = cudaMalloc(&d->fields, at + sizeof(DevCounters));
+    if (e == cudaSuccess) d->counters = reinterpret_cast<DevCounters*>(static_cast<char*>(d->fields) + at);
     if (e == cudaSuccess) e = cudaMallocHost(&d->host_counters, sizeof(DevCounters));
     if (e == cudaSuccess)
         e = cudaMemcpyAsync(d->cells, cells.data(), sizeof(D4) * cells.size(), cudaMemcpyHostToDevice, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d->fields, 0, d->field_bytes, s);
-    if (e == cudaSuccess) e = cudaMemsetAsync(d->counters, 0, sizeof(DevCounters), s);
+    if (e == cudaSuccess) e = cudaMemsetAsync(d->fields, 0, at + sizeof(DevCounters), s);
     if (e == cudaSuccess) e = cudaStreamSynchronize(s);
     if (e != cudaSuccess) {
         rd_status st = cuda_fail(e, "rd_create_detector");
         cudaFree(d->cells);
         cudaFree(d->fields);
-        cudaFree(d->counters);
         cudaFreeHost(d->host_counters);
         delete d;
         return st;
@@ -444,7 +447,6 @@ rd_status rd_destroy(rd_detector* d)
     for (auto& ev : d->ev_free) { cudaEventDestroy(ev.first); cudaEventDestroy(ev.second); }
     cudaFree(d->cells);
     cudaFree(d->fields);
-    cudaFree(d->counters);
     cudaFreeHost(d->host_counters);
     cudaFree(d->rec);
     cudaFree(d->stage);
@@ -467,8 +469,10 @@ rd_status rd_zero_fields(rd_detector* d, rd_stream stream)
     g_err.clear();
     if (!d) return fail(RD_ERR_ARG, "detector is NULL");
     cudaStream_t s = reinterpret_cast<cudaStream_t>(stream);
-    RD_CUDA(cudaMemsetAsync(d->fields, 0, d->field_bytes, s), "rd_zero_fields");
-    RD_CUDA(cudaMemsetAsync(&d->counters->clipped, 0, 2 * sizeof(unsigned long long), s), "rd_zero_fields");
+    // the fields and the two counts behind them (not the latched errors)
+    static_assert(offsetof(DevCounters, errors) == 2 * sizeof(unsigned long long), "counts first");
+    RD_CUDA(cudaMemsetAsync(d->fields, 0, counters_at(d->field_bytes) + offsetof(DevCounters, errors), s),
+            "rd_zero_fields");
     d->n_deposits = 0;
     return RD_OK;
 }

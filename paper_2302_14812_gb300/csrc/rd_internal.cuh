@@ -29,10 +29,10 @@ enum : unsigned {
 };
 
 struct DevCounters {
-    unsigned errors;
-    unsigned pad;
     unsigned long long clipped;
     unsigned long long crossings;   // bin edges crossed by arrival intervals (mixed path)
+    unsigned errors;                // (last: the two counts are cleared together with the fields)
+    unsigned pad;
 };
 
 // ---------------------------------------------------------------------------------------------
