@@ -96,6 +96,31 @@ __device__ __forceinline__ df2 df_fma(df2 a, df2 b, df2 c)
     return fast_two_sum(s.hi, t);
 }
 
+// Products and sums without the last renormalisation (|lo| up to a few ulp(hi)): for results that only enter
+// another sum or product, which keeps its error within a few units of 2^-47.
+__device__ __forceinline__ df2 df_mul_u(df2 a, df2 b)
+{
+    df2 p = two_prod(a.hi, b.hi);
+    p.lo = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
+    return p;
+}
+
+__device__ __forceinline__ df2 df_fma_u(df2 a, df2 b, df2 c)
+{
+    const df2 p = two_prod(a.hi, b.hi);
+    df2 s = two_sum(p.hi, c.hi);
+    const float t = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
+    s.lo = __fadd_rn(t, __fadd_rn(c.lo, s.lo));
+    return s;
+}
+
+__device__ __forceinline__ df2 df_add_u(df2 a, df2 b)
+{
+    df2 s = two_sum(a.hi, b.hi);
+    s.lo = __fadd_rn(s.lo, __fadd_rn(a.lo, b.lo));
+    return s;
+}
+
 // 1 / a: y = rcp.approx(hi), e = 1 - a y (the fused multiply-add makes 1 - hi y exact to its own
 // rounding), result y + y e
 __device__ __forceinline__ df2 df_rcp(df2 a)
