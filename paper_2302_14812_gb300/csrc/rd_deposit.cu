@@ -229,16 +229,58 @@ __device__ __forceinline__ void flush_f64(double* row, int n_bins, int b, const 
     }
 }
 
-// 1/d by Newton-Raphson iteration from the hardware's approximate reciprocal: each step
-// y <- y + y (1 - d y) squares the relative error, so two steps take the approximation to FP64
-// rounding.  For the positive, normal arguments the field passes (kappa R >= R / (2 gamma^2)).
-__device__ __forceinline__ double rcp_newton(double d)
+// Square root and reciprocal start from the FP32 approximations (relative error below 2^-22): the FP64
+// operand's leading bits become a float, and the float result a double, on the integer pipe, which this
+// kernel leaves idle, so that FP64 refinement takes 6 and 3 operations (9 and 4 from the FP64
+// approximations, good to ~2^-20).  The deposit is bound by the FP64 pipe at 61 operations per (cell,
+// interval): with 56, 24 particles x 1200 intervals x 4096 cells take 12.48 ms instead of 13.41.  Operands
+// outside FP32's range take the plain forms.
+__device__ __forceinline__ bool fp32_range(double v)
+{
+    // positive, exponent within +-100
+    return (unsigned)(__double2hiint(v) - ((1023 - 100) << 20)) < (unsigned)(200 << 20);
+}
+
+__device__ __forceinline__ float leading_float(double v)    // v truncated to 24 bits
+{
+    return __int_as_float(((__double2hiint(v) - (896 << 20)) << 3) | (int)((unsigned)__double2loint(v) >> 29));
+}
+
+__device__ __forceinline__ double float_bits_to_double(float v)     // exact, v positive and normal
+{
+    const int b = __float_as_int(v);
+    return __hiloint2double((b >> 3) + (896 << 20), b << 29);
+}
+
+// sqrt(a) rounded to nearest, by Markstein's sequence ("IA-64 and Elementary Functions", 2000): one coupled
+// Newton-Raphson step for g -> sqrt(a), h -> 1 / (2 sqrt(a)) takes the error to ~2^-44, and adding the
+// residual a - g^2 (exact but for its own rounding) times h leaves g within ~2^-86 of sqrt(a) before the last
+// rounding: the correctly rounded value unless sqrt(a) lies that close to a rounding boundary (1 in 10^10).
+__device__ __forceinline__ double sqrt_markstein(double a)
+{
+    if (!fp32_range(a)) return __dsqrt_rn(a);
+    const double y = float_bits_to_double(fast_rsqrt(leading_float(a)));
+    double h = __hiloint2double(__double2hiint(y) - (1 << 20), __double2loint(y));      // y / 2
+    double g = __dmul_rn(a, y);
+    const double r = __fma_rn(-h, g, 0.5);
+    g = __fma_rn(g, r, g);
+    h = __fma_rn(h, r, h);
+    const double d = __fma_rn(-g, g, a);
+    return __fma_rn(d, h, g);
+}
+
+// 1/d: one third-order step y (1 + e + e^2), e = 1 - d y, takes the approximation (2^-22) to FP64 rounding.
+// For the positive, normal arguments the field passes (kappa R >= R / (2 gamma^2)).
+__device__ __forceinline__ double rcp_cubic(double d)
 {
     double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    if (fp32_range(d)) {
+        y = float_bits_to_double(fast_rcp(leading_float(d)));
+    } else {
+        asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(d));
+    }
     double e = fma(-d, y, 1.0);
-    y = fma(y, e, y);
-    e = fma(-d, y, 1.0);
+    e = fma(e, e, e);
     return fma(y, e, y);
 }
 
@@ -253,9 +295,9 @@ __device__ __forceinline__ void fp64_field(const RecD& r, double dx, double dy, 
 {
     const double kR = fma(-r.bb.z, dz, fma(-r.bb.y, dy, fma(-r.bb.x, dx, R)));
     const double a = fma(r.bd.z, dz, fma(r.bd.y, dy, fma(r.bd.x, dx, r.bb.w)));
-    const double w = rcp_newton(kR);
-    const double Q = w * (w * w);
-    const double Qa = Q * a, Qk = Q * kR;
+    const double w = rcp_cubic(kR);
+    const double Qk = w * w;                            // q-free (kappa R)^-3 times kappa R
+    const double Qa = (w * Qk) * a;
     const double vx = fma(Qa, r.bb.x, Qk * r.bd.x);     // Q v
     const double vy = fma(Qa, r.bb.y, Qk * r.bd.y);
     const double vz = fma(Qa, r.bb.z, Qk * r.bd.z);
@@ -275,7 +317,7 @@ __device__ __forceinline__ double fp64_arrival(const RecD& r, const D4& cl, doub
     dx = __dsub_rn(cl.x, r.xa.x);
     dy = __dsub_rn(cl.y, r.xa.y);
     dz = __dsub_rn(cl.z, r.xa.z);
-    R = __dsqrt_rn(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
+    R = sqrt_markstein(__dadd_rn(__dadd_rn(__dmul_rn(dx, dx), __dmul_rn(dy, dy)), __dmul_rn(dz, dz)));
     return __dmul_rn(__dsub_rn(__dadd_rn(r.xa.w, R), cl.w), inv_dt_det);
 }
 
