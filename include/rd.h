@@ -320,8 +320,8 @@ RD_API rd_status rd_set_batch_budget(rd_detector* det, long long bytes);
 
 /*
  * Steps per work item (the step chunk between exact FP64 arrival anchors) for this detector's
- * deposits; 0 = automatic (equal chunks of at most 2048; where the work makes few waves of CTAs, the
- * split, down to 16 intervals, that finishes them soonest).
+ * deposits; 0 = automatic (RD_MIXED: 2048, halved while the grid would be too small to fill the GPU; RD_FP64:
+ * equal chunks of at most 2048, where the work makes few waves of CTAs the split that finishes them soonest).
  */
 RD_API rd_status rd_set_chunk(rd_detector* det, int32_t chunk);
 

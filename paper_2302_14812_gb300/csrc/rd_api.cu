@@ -154,11 +154,11 @@ rd_status check_traj(const rd_traj* t)
     return RD_OK;
 }
 
-// Intervals per work item: the detector's override, else the default rule for the detector's kernel.
-int choose_chunk(const rd_detector* d, int n_part, int S, int n_cell_blocks, int per_sm)
+// Intervals per work item: the detector's override, else the default rule of the detector's kernel.
+int choose_chunk(const rd_detector* d, int n_part, int S, int n_cell_blocks)
 {
     if (d->chunk_override > 0) return std::min(d->chunk_override, S);
-    return auto_chunk(n_cell_blocks, n_part, S, per_sm, d->precision == RD_MIXED ? kMixedSetup : kFp64Setup);
+    return d->precision == RD_MIXED ? auto_chunk(n_cell_blocks, n_part, S) : wave_chunk(n_cell_blocks, n_part, S);
 }
 
 // Bracket one deposit-kernel launch with events when timing is on.
@@ -261,16 +261,24 @@ int grid_stride_blocks(long long n, int threads, int per_sm)
     return (int)std::max(1LL, g);
 }
 
-int auto_chunk(long long n_cell_blocks, long long n_part, int S, int per_sm, int setup)
+int auto_chunk(long long n_cell_blocks, long long n_part, int S)
 {
-    const long long R = (long long)sm_count() * per_sm, base = n_cell_blocks * n_part;
+    int chunk = std::min(kDefaultChunk, S);
+    const long long want = 8LL * sm_count();       // resident CTAs for a few waves
+    while (chunk > 64 && n_cell_blocks * n_part * ((S + chunk - 1) / chunk) < want) chunk /= 2;
+    return std::max(1, chunk);
+}
+
+int wave_chunk(long long n_cell_blocks, long long n_part, int S)
+{
+    const long long R = (long long)sm_count() * kFp64CtasPerSm, base = n_cell_blocks * n_part;
     const long long n_min = (S + kDefaultChunk - 1) / kDefaultChunk;            // chunks of a trajectory
     const long long n_max = std::max<long long>(n_min, S / kMinChunk);
     auto chunk_of = [&](long long n) { return (int)((S + n - 1) / n); };
     int best = std::max(1, chunk_of(std::max(1LL, n_min)));
     auto cost = [&](int chunk) {
         const long long items = base * ((S + chunk - 1) / chunk);
-        return ((items + R - 1) / R) * (long long)(chunk + setup);
+        return ((items + R - 1) / R) * (long long)(chunk + kFp64Setup);
     };
     if (base > 0 && base * n_min <= kMaxWaves * R) {
         for (long long w = 1; w <= kMaxWaves; ++w) {                            // most chunks within w waves
@@ -507,8 +515,7 @@ static rd_status deposit_from(rd_detector* d, const rd_traj* t, rd_stream stream
     const int cpc = def_shape ? kMixedCellsPerCta : d->cpc, nc = def_shape ? kMixedCells : d->nc;
     static_assert(kDepositThreads == kMixedCellsPerCta, "both deposit kernels cover 256 cells per CTA");
     const int n_cell_blocks = (d->n_pix + (mixed ? cpc : kDepositThreads) - 1) / (mixed ? cpc : kDepositThreads);
-    const int per_sm = mixed ? mixed_ctas_per_sm(cpc, nc, d->flags) : kFp64CtasPerSm;
-    const int chunk = choose_chunk(d, std::min(pc, t->n_part), S - k_first + 1, n_cell_blocks, per_sm);
+    const int chunk = choose_chunk(d, std::min(pc, t->n_part), S - k_first + 1, n_cell_blocks);
 
     for (int p0 = 0; p0 < t->n_part; p0 += pc) {
         const int np = std::min(pc, t->n_part - p0);
@@ -1078,12 +1085,9 @@ rd_status rd_deposit_batch(int32_t n, rd_detector* const* dets, const rd_traj* t
         const size_t per_part = sizeof(RecS) * (size_t)t.n_samples;
         const size_t budget = std::max(d0->batch_budget, per_part);
         const int ncb = (dets[i]->n_pix + kMixedCellsPerCta - 1) / kMixedCellsPerCta;
-        // (chunks of equal length: a last chunk much shorter than the others pays the same set-up)
-        const int n_cap = (S + cap - 1) / cap;
         const int chunk = full_chunks ? (dets[i]->chunk_override > 0 ? std::min(dets[i]->chunk_override, S)
-                                                                      : (S + n_cap - 1) / n_cap)
-                                      : choose_chunk(dets[i], t.n_part, S, ncb,
-                                                     mixed_ctas_per_sm(kMixedCellsPerCta, kMixedCells, dets[i]->flags));
+                                                                      : std::min(cap, S))
+                                      : choose_chunk(dets[i], t.n_part, S, ncb);
         for (int p0 = 0; p0 < t.n_part;) {
             if (budget - std::min(used, budget) < per_part && group_first.back() != (int)segs.size()) {
                 group_first.push_back((int)segs.size());           // close the group

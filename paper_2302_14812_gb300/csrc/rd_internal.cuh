@@ -169,26 +169,23 @@ struct PrecomputeGrid {
         blocks = (unsigned)((warps * 32 + threads - 1) / threads);
     }
 };
-// Default intervals per work item of a deposit launch: its cell blocks x particles x chunks run in waves of
-// the per_sm CTAs a multiprocessor holds, and an item costs its intervals plus `setup` (anchors and first
-// records, in intervals' time).  Chunks are of equal length, at most kDefaultChunk; while that makes few
-// waves (at most kMaxWaves), the split of the trajectory into more chunks that minimises waves x (chunk +
-// setup) is taken, down to kMinChunk intervals.  Measured against halving 2048 until the grid held 8 CTAs
-// per multiprocessor (unequal last chunks, half-empty last waves): FP64, 24 particles x 1200 intervals x
-// 4096 cells 14.33 -> 13.41 ms (5.05 waves of 300 intervals -> 8.8 of 172); mixed, 37 x 3001 x 3233
-// 0.873 -> 0.832 ms, 1 x 2000 x 64 cells 19 -> 11 us.  The set-up figures hold to a factor of two: 30 or
-// 100 intervals for the mixed kernel change these by less than 1.5 %.
+// Default intervals per work item of the mixed deposit: kDefaultChunk (at most S), halved while the grid (cell
+// blocks x particles x chunks) would hold fewer than 8 CTAs per multiprocessor.  (The FP32 walk's drift shows
+// where a chunk ends: its last interval closes the gap to the FP64 anchor.  On pulses much shorter than a
+// bin's worth of steps -- gamma 5 circular orbits -- that is 3e-5 of the fields' norm, so the chunk ends stay
+// where they are; filling the last wave better, as below, gave 0 to 5 %.)
+int auto_chunk(long long n_cell_blocks, long long n_part, int S);
+// The same of the FP64 deposit, whose result does not depend on the chunks beyond the order of its sums: the
+// work runs in waves of the CTAs the multiprocessors hold, and an item costs its intervals plus kFp64Setup
+// (anchors and first records, in intervals' time).  Equal chunks of at most kDefaultChunk; while that makes
+// few waves (at most kMaxWaves), the split of the trajectory that minimises waves x (chunk + set-up), down to
+// kMinChunk intervals.  24 particles x 1200 intervals x 4096 cells: 14.33 ms by the halving rule (5.05 waves
+// of 300 intervals), 13.41 ms (8.8 of 172).
 constexpr int kMaxWaves = 16;
 constexpr int kMinChunk = 16;
-#ifndef RD_MIXED_SETUP
-#define RD_MIXED_SETUP 60
-#endif
-constexpr int kMixedSetup = RD_MIXED_SETUP;
 constexpr int kFp64Setup = 5;
 constexpr int kFp64CtasPerSm = 2;
-int auto_chunk(long long n_cell_blocks, long long n_part, int S, int per_sm, int setup);
-// CTAs per multiprocessor of the mixed kernel of a shape and a detector's flags
-int mixed_ctas_per_sm(int cells_per_cta, int cells_per_thread, int flags);
+int wave_chunk(long long n_cell_blocks, long long n_part, int S);
 // Cell blocks per group of the mixed kernels' work order (item_coords): as many as keep the group's
 // active detector slice (cells_per_cta x 32 bytes x the bins a step chunk of `chunk` of the
 // trajectory's n_intervals spans, per block) within RD_GROUP_SLICE_MB, at most 8.

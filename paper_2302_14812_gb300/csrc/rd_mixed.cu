@@ -1427,12 +1427,6 @@ static void launch_mixed(const DepositParams& p, unsigned blocks, cudaStream_t s
     k_deposit_mixed<FF, LIN, NC, CPC><<<blocks, CPC / NC, 0, s>>>(p);
 }
 
-int mixed_ctas_per_sm(int cells_per_cta, int cells_per_thread, int flags)
-{
-    const int lin = (flags & RD_QUADRATIC) ? 2 : (flags & (RD_LINEAR | RD_HOLD_PREV)) ? 1 : 0;
-    return mixed_min_blocks(cells_per_cta / cells_per_thread, (flags & RD_FARFIELD) != 0, lin);
-}
-
 bool mixed_shape_supported(int cells_per_cta, int cells_per_thread)
 {
     return (cells_per_cta == 64 || cells_per_cta == 128 || cells_per_cta == 256) &&

@@ -115,8 +115,7 @@ extern "C" rd_status rd_deposit_noalloc(const double* pix_pos, const double* pix
     if (e == cudaSuccess && t->n_part > 0 && S >= 1) {
         const int pc = (int)std::max<size_t>(1, std::min<size_t>((size_t)t->n_part, kRecordBytes / per_part));
         const int n_cell_blocks = (n_pix + kMixedCellsPerCta - 1) / kMixedCellsPerCta;
-        const int chunk = auto_chunk(n_cell_blocks, std::min(pc, t->n_part), S,
-                                     mixed_ctas_per_sm(kMixedCellsPerCta, kMixedCells, fl), kMixedSetup);
+        const int chunk = auto_chunk(n_cell_blocks, std::min(pc, t->n_part), S);
         for (int p0 = 0; p0 < t->n_part && e == cudaSuccess; p0 += pc) {
             const int np = std::min(pc, t->n_part - p0);
             const size_t off = (size_t)p0 * t->n_samples * 3;
