@@ -48,7 +48,7 @@ def _deposit(tr, det, nc=None):
     import torch
     d = rd.RadiationDetector.from_workload(det, "mixed")
     if nc is not None:
-        d.set_shape(256, nc, tr.n_steps, 1)
+        d.set_shape(128, nc, tr.n_steps, 1)     # (a small grid of the default 256 x 2 runs one cell per thread)
     d.deposit(torch.from_numpy(tr.x).cuda(), torch.from_numpy(tr.u).cuda(), torch.from_numpy(tr.q).cuda(), tr.t0, tr.dt)
     E, B = d.read("float32")
     st = d.stats()
@@ -97,3 +97,18 @@ def test_runs_of_bins(n_steps, width, flags):
     d.close()
     assert st.n_clipped == clipped and st.device_errors == 0
     assert parity_err(E, Eo) <= 1e-4 and parity_err(B, Bo) <= 1e-4
+
+
+@pytest.mark.parametrize("n_cells", [1, 63, 64, 65, 256, 257, 700])
+def test_small_grids_run_one_cell_per_thread(n_cells):
+    """The default shape on a small grid against the two-cell shape it stands in for."""
+    tr, det = _case(130, 1.1)
+    det = W.Detector(np.resize(det.pix_pos, (n_cells, 3)), np.resize(det.pix_t0, n_cells), 0.0, det.dt_det, det.n_bins)
+    E2, B2 = _deposit(tr, det, 2)
+    import torch
+    d = rd.RadiationDetector.from_workload(det, "mixed")
+    d.set_chunk(tr.n_steps)
+    d.deposit(torch.from_numpy(tr.x).cuda(), torch.from_numpy(tr.u).cuda(), torch.from_numpy(tr.q).cuda(), tr.t0, tr.dt)
+    E, B = d.read("float32")
+    d.close()
+    assert np.array_equal(E, E2) and np.array_equal(B, B2)
