@@ -1219,13 +1219,14 @@ rd_status rd_power_spectrum(rd_detector* d, int32_t which, float* out, rd_stream
     if (st != RD_OK) return st;
     const int M = spectrum_twiddle_length(N);
     if (d->spec_n != N) {
-        st = ensure(&d->spec_tw, &d->spec_tw_bytes, sizeof(float2) * (M / 2), s, "twiddles");
+        const bool rem = spectrum_split(N);
+        const size_t len = rem ? M : M / 2;
+        st = ensure(&d->spec_tw, &d->spec_tw_bytes, sizeof(float2) * len, s, "twiddles");
         if (st != RD_OK) return st;
         RD_CUDA(cudaStreamSynchronize(s), "twiddles");          // the host table may be in flight
-        d->spec_tw_host.resize(M / 2);
-        fill_twiddles(d->spec_tw_host.data(), M);
-        RD_CUDA(cudaMemcpyAsync(d->spec_tw, d->spec_tw_host.data(), sizeof(float2) * (M / 2), cudaMemcpyHostToDevice,
-                                s),
+        d->spec_tw_host.resize(len);
+        fill_twiddles(d->spec_tw_host.data(), M, rem);
+        RD_CUDA(cudaMemcpyAsync(d->spec_tw, d->spec_tw_host.data(), sizeof(float2) * len, cudaMemcpyHostToDevice, s),
                 "twiddles");
         d->spec_n = N;
     }

@@ -291,11 +291,13 @@ cudaError_t launch_read_fields(const void* fields, int precision, int n_pix, int
                                void* B, int dtype, cudaStream_t s);
 cudaError_t launch_write_fields(void* fields, int precision, int n_pix, int n_bins, const void* E, const void* B,
                                 int dtype, cudaStream_t s);
-// power spectra (rd_spectrum.cu): twiddles exp(-2 pi i j / N), j < N/2, computed on the host
-void fill_twiddles(float2* host, int N);
+// power spectra (rd_spectrum.cu): twiddles exp(-2 pi i j / M), j < M / 2, computed on the host; then, where
+// asked for, what rounding each to FP32 left out
+void fill_twiddles(float2* host, int M, bool remainders);
 constexpr int kFusedMaxN = 8192;   // longest series transformed in shared memory (24.5 N bytes per CTA)
 constexpr int kSplitMaxN = 1 << 22;  // longest series transformed as columns, then rows
 bool spectrum_fused(int N);
+bool spectrum_split(int N);                       // transformed as columns, then rows (its table has remainders)
 int spectrum_twiddle_length(int N);               // twiddle table of a length-N series: exp(-2 pi i j / M), j < M / 2
 size_t spectrum_work_bytes(int n_pix, int N);
 cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* work,

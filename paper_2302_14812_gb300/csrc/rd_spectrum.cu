@@ -135,12 +135,35 @@ __device__ __forceinline__ float2 mul_root16(float2 a, int j)
     return cmul(a, root16(j));
 }
 
+// The same product with the roots to twice FP32's digits (hi + lo, both rounded from the exact values):
+// the lo parts are added to the smaller product before its rounding, so only the two roundings of an
+// exact root's product remain.
+__device__ __forceinline__ float2 mul_root16_comp(float2 a, int j)
+{
+    if (j == 0) return a;
+    if (j == 4) return make_float2(a.y, -a.x);
+    constexpr double c1 = 0.92387953251128674, s1 = 0.38268343236508978, h = 0.70710678118654752;
+    if (j == 2 || j == 6) {             // (+-1 - i) / sqrt 2
+        const float hh = (float)h, hl = (float)(h - (double)(float)h);
+        const float u = a.x + a.y, v = a.y - a.x;
+        const float hu = __fmaf_rn(u, hh, __fmul_rn(u, hl)), hv = __fmaf_rn(v, hh, __fmul_rn(v, hl));
+        return j == 2 ? make_float2(hu, hv) : make_float2(hv, -hu);
+    }
+    constexpr double re[8] = {1., c1, h, s1, 0., -s1, -h, -c1}, im[8] = {0., -s1, -h, -c1, -1., -c1, -h, -s1};
+    const float rh = (float)re[j], rl = (float)(re[j] - (double)rh);
+    const float ih = (float)im[j], il = (float)(im[j] - (double)ih);
+    const float x = __fmaf_rn(a.y, ih, __fmaf_rn(a.y, il, -__fmul_rn(a.x, rl)));
+    const float y = __fmaf_rn(a.y, rh, __fmaf_rn(a.y, rl, __fmul_rn(a.x, il)));
+    return make_float2(__fmaf_rn(a.x, rh, -x), __fmaf_rn(a.x, ih, y));
+}
+
 // In-register DFT of length R (2, 4, 8, 16): X[k] = sum_r a[r] exp(-2 pi i r k / R), by radix-2
 // decimation in frequency; the result is left in bit-reversed order (a[bitrev(k)] = X[k]).
+// COMP: with the roots to twice FP32's digits.
 template <int R>
 constexpr int log2_of() { return R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1; }
 
-template <int R>
+template <int R, bool COMP = false>
 __device__ __forceinline__ void dft_bitrev(float2 (&a)[R])
 {
     constexpr int L = log2_of<R>();
@@ -154,7 +177,8 @@ __device__ __forceinline__ void dft_bitrev(float2 (&a)[R])
                 const int j = g * (R >> st);
                 const float2 u = a[j + i], v = a[j + i + h];
                 a[j + i] = cadd(u, v);
-                a[j + i + h] = mul_root16(csub(u, v), i * (8 / h));     // exp(-2 pi i i / (2h))
+                const float2 d = csub(u, v);                    // times exp(-2 pi i i / (2h))
+                a[j + i + h] = COMP ? mul_root16_comp(d, i * (8 / h)) : mul_root16(d, i * (8 / h));
             }
         }
     }
@@ -220,8 +244,8 @@ __device__ __forceinline__ void spec_pass(float2* z1, float2* z2, const T* row, 
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
         if (!on[u]) continue;
-        dft_bitrev<R>(a1[u]);
-        dft_bitrev<R>(a2[u]);
+        dft_bitrev<R, true>(a1[u]);
+        dft_bitrev<R, true>(a2[u]);
         const int o = bq[u] + s * R * bp[u];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -335,14 +359,46 @@ cudaError_t launch_fused(const T* fields, int n_pix, int N, int c0, const float2
 // read again for Y, 2 written for the power.  Cells go through both kernels in batches whose Y fits L2, so
 // only the bins and the power touch DRAM.  Measured, 512 cells x 131072 bins: 6.12 ms as 17 radix-2 passes
 // over the batch (4.3 GB each) plus packing and power; 0.90 ms in two kernels per batch of 42 cells (columns
-// 0.52 ms, 4.1 TB/s of the bins; rows 0.38 ms).
+// 0.52 ms, 4.1 TB/s of the bins; rows 0.38 ms).  The fixed roots of the in-register transforms and the roots
+// between the kernels carry FP32's remainders: every butterfly multiplies by the same few roots, so their
+// rounding adds up where radix-2 passes average over a table.  Relative L2 error of the power of noise
+// against FP64, N = 2^14 / 2^17 / 2^22: radix-2 passes 1.29 / 1.38 / 1.50e-7, here 1.15 / 1.19 / 1.32e-7, and
+// 1.66 / 1.82 / 2.12e-7 with roots rounded to FP32, at the same speed (bound by memory).
 // ---------------------------------------------------------------------------------------------
 constexpr int kColumnElems = 4096;      // elements of each of Z1, Z2 per CTA of k_split_columns, 16 per thread
 constexpr int kColumnThreads = kColumnElems / 16;
 
+// a (h + l) for a root h of FP32 digits and its small remainder l: the remainder joins the smaller product
+// before its rounding.
+__device__ __forceinline__ float2 cmul_comp(float2 a, float2 h, float2 l)
+{
+    const float x = __fmaf_rn(a.y, h.y, __fmaf_rn(a.y, l.y, -__fmul_rn(a.x, l.x)));
+    const float y = __fmaf_rn(a.y, h.x, __fmaf_rn(a.y, l.x, __fmul_rn(a.x, l.y)));
+    return make_float2(__fmaf_rn(a.x, h.x, -x), __fmaf_rn(a.x, h.y, y));
+}
+
+// h and l with h + l = exp(-2 pi i e / N), e < N: h the table's root exp(-2 pi i j / N1) at the nearest multiple
+// j of N / N1 = N2, l = its lo part plus h (exp(-i theta) - 1), |theta| <= pi / N1 < 0.1, by the power series
+// (the first terms left out are theta^7 / 5040 < 2e-11 and theta^8 / 40320).  (sincospif's value is off by up
+// to an ulp, which the transform's error showed.)
+template <int N1>
+__device__ __forceinline__ void split_root(const float2* tw, int e, int N2, float two_over_n, float2& h, float2& l)
+{
+    const int log2_n2 = 31 - __clz(N2), j = (e + N2 / 2) >> log2_n2;
+    const float th = 3.14159265358979f * (two_over_n * (float)(e - (j << log2_n2))), t2 = th * th;
+    const float sn = th * (1.f - t2 * (1.f / 6.f - t2 * (1.f / 120.f)));
+    const float vc = t2 * (0.5f - t2 * (1.f / 24.f - t2 * (1.f / 720.f)));          // 1 - cos
+    const bool neg = j & (N1 / 2);
+    const int i = j & (N1 / 2 - 1);
+    const float2 a = tw[i], b = tw[N1 / 2 + i];
+    h = neg ? make_float2(-a.x, -a.y) : a;
+    const float2 lo = neg ? make_float2(-b.x, -b.y) : b;
+    l = make_float2(lo.x + (h.y * sn - h.x * vc), lo.y - (h.x * sn + h.y * vc));
+}
+
 // One Stockham pass (see spec_pass) of radix R at stride S over the columns of both transforms, rows of
 // C elements in shared memory (row i at pad(i)); LAST: the results go to global memory, multiplied by
-// exp(-2 pi i n2 k1 / N).  tw: exp(-2 pi i j / N1), j < N1 / 2.
+// exp(-2 pi i n2 k1 / N).  tw: exp(-2 pi i j / N1), j < N1 / 2, rounded to FP32, then the remainders.
 template <int N1, int S, typename T, int STRIDE>
 __device__ __forceinline__ void column_passes(float2* z1, float2* z2, const float2* tw, const T* row, int c0, int N2,
                                               int n2, float two_over_n, float2* Y1, float2* Y2)
@@ -372,19 +428,18 @@ __device__ __forceinline__ void column_passes(float2* z1, float2* z2, const floa
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
         const int b = t + u * (N1 / 16), q = b % S, p = b / S;
-        dft_bitrev<R>(a1[u]);
-        dft_bitrev<R>(a2[u]);
+        dft_bitrev<R, true>(a1[u]);
+        dft_bitrev<R, true>(a2[u]);
         const int o = q + S * R * p;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             float2 b1 = a1[u][bitrev<R>(k)], b2 = a2[u][bitrev<R>(k)];
             const int i = o + S * k;
             if (LAST) {                 // m = 1, p = 0: no twiddle of its own; i = k1
-                float sn, cs;
-                sincospif(two_over_n * (float)(i * n2), &sn, &cs);      // exact argument: i n2 < N <= 2^22
-                const float2 w = make_float2(cs, -sn);
-                Y1[(size_t)i * N2 + n2] = cmul(b1, w);
-                if (i <= N1 / 2) Y2[(size_t)i * N2 + n2] = cmul(b2, w);
+                float2 wh, wl;
+                split_root<N1>(tw, i * n2, N2, two_over_n, wh, wl);
+                Y1[(size_t)i * N2 + n2] = cmul_comp(b1, wh, wl);
+                if (i <= N1 / 2) Y2[(size_t)i * N2 + n2] = cmul_comp(b2, wh, wl);
             } else {
                 if (k > 0) {
                     const float2 w = twiddle(tw, p * k * S, N1 / 2);
@@ -404,10 +459,10 @@ __device__ __forceinline__ void column_passes(float2* z1, float2* z2, const floa
 
 constexpr size_t split_columns_smem(int N1)
 {
-    return sizeof(float2) * (2 * (size_t)(N1 + N1 / 16) * (kColumnElems / N1) + N1 / 2);
+    return sizeof(float2) * (2 * (size_t)(N1 + N1 / 16) * (kColumnElems / N1) + N1);
 }
 
-// grid (N2 / C, cells); tab: exp(-2 pi i j / M), j < M / 2, M = N1 tab_step
+// grid (N2 / C, cells); tab: exp(-2 pi i j / M), j < M / 2, M = N1 tab_step, rounded to FP32, then the remainders
 template <int N1, typename T, int STRIDE>
 __global__ void __launch_bounds__(kColumnThreads, 2) k_split_columns(const T* __restrict__ fields, int c0, int N2,
                                                                      const float2* __restrict__ tab, int tab_step,
@@ -416,7 +471,7 @@ __global__ void __launch_bounds__(kColumnThreads, 2) k_split_columns(const T* __
     extern __shared__ float2 sm[];
     constexpr int C = kColumnElems / N1, zlen = (N1 + N1 / 16) * C;
     float2* tw = sm + 2 * zlen;
-    for (int j = threadIdx.x; j < N1 / 2; j += kColumnThreads) tw[j] = tab[j * tab_step];
+    for (int j = threadIdx.x; j < N1; j += kColumnThreads) tw[j] = tab[j * tab_step];       // (the halves of tab too)
     __syncthreads();
     const size_t cell = blockIdx.y;
     const int n2 = blockIdx.x * C + threadIdx.x % C;
@@ -449,7 +504,7 @@ __device__ __forceinline__ void row_passes(float2* const (&z)[3], const float2* 
         const int b = t + u * (N2 / 16), q = b % S, p = b / S;
         const int o = q + S * R * p;
 #pragma unroll
-        for (int v = 0; v < 3; ++v) dft_bitrev<R>(a[v][u]);
+        for (int v = 0; v < 3; ++v) dft_bitrev<R, true>(a[v][u]);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float2 w = (m > 1 && k > 0) ? twiddle(tw, p * k * S, N2 / 2) : make_float2(1.f, 0.f);
@@ -579,17 +634,18 @@ int grid_for(long long n, int threads) { return grid_stride_blocks(n, threads, 3
 
 }  // namespace
 
-void fill_twiddles(float2* host, int N)
+void fill_twiddles(float2* host, int M, bool remainders)
 {
     const double two_pi = 6.283185307179586476925287;
-    for (int j = 0; j < N / 2; ++j) {
-        const double a = -two_pi * (double)j / (double)N;
-        host[j] = make_float2((float)cos(a), (float)sin(a));
+    for (int j = 0; j < M / 2; ++j) {
+        const double a = -two_pi * (double)j / (double)M, c = cos(a), s = sin(a);
+        host[j] = make_float2((float)c, (float)s);
+        if (remainders) host[M / 2 + j] = make_float2((float)(c - (double)host[j].x), (float)(s - (double)host[j].y));
     }
 }
 
 bool spectrum_fused(int N) { return N >= 2 && N <= kFusedMaxN; }
-static bool spectrum_split(int N) { return N > kFusedMaxN && N <= kSplitMaxN; }
+bool spectrum_split(int N) { return N > kFusedMaxN && N <= kSplitMaxN; }
 
 int spectrum_twiddle_length(int N)
 {
@@ -606,7 +662,8 @@ size_t spectrum_work_bytes(int n_pix, int N)
     return 2 * sizeof(float2) * 2 * (size_t)n_pix * N;
 }
 
-// work: spectrum_work_bytes; tw: exp(-2 pi i j / M), j < M / 2, M = spectrum_twiddle_length(N).
+// work: spectrum_work_bytes; tw: exp(-2 pi i j / M), j < M / 2, M = spectrum_twiddle_length(N) (split
+// transforms: then the M / 2 remainders of rounding them to FP32).
 cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, int N, int c0, float2* work,
                                   const float2* tw, float scale, float* P, cudaStream_t s)
 {

@@ -36,3 +36,34 @@ def test_long_series(log2n, n_pix, precision):
         assert P.shape == ref.shape
         assert parity_err(P, ref) <= 1e-5
     d.close()
+
+
+def _radix2(x):
+    """Stockham radix-2 transform in complex64, roots rounded from FP64."""
+    n, s, size = x.shape[-1], 1, x.shape[-1]
+    while n > 1:
+        i = np.arange(size // 2)
+        p, q = i // s, i % s
+        w = np.exp(-2j * np.pi * p / n).astype(np.complex64)
+        a, b = x[..., : size // 2], x[..., size // 2:]
+        y = np.empty_like(x)
+        y[..., q + 2 * s * p] = a + b
+        y[..., q + 2 * s * p + s] = (a - b) * w
+        x, n, s = y, n // 2, 2 * s
+    return x
+
+
+@pytest.mark.parametrize("log2n", [14, 17, 19, 20])
+def test_error_no_larger_than_radix2(log2n):
+    """The columns-and-rows transform is no less accurate than log2 N radix-2 passes in FP32."""
+    n, n_pix = 1 << log2n, 4
+    rng = np.random.default_rng(100 + log2n)
+    f = rng.normal(size=(n_pix, n, 3)).astype(np.float32)
+    d = rd.RadiationDetector(rng.normal(size=(n_pix, 3)) + 30.0, 0.0, 1.0, n, precision="mixed")
+    d.write(f, f)
+    P = d.power_spectrum("E").cpu().numpy().astype(np.float64)
+    d.close()
+    ref = np.sum(np.abs(np.fft.rfft(f.astype(np.float64), axis=1)) ** 2, axis=2)
+    plain = np.sum(np.abs(_radix2(np.moveaxis(f, 1, 2).astype(np.complex64))[..., : n // 2 + 1].astype(np.complex128)) ** 2,
+                   axis=1)
+    assert np.linalg.norm(P - ref) <= np.linalg.norm(plain - ref)
