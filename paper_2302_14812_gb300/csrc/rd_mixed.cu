@@ -839,13 +839,17 @@ __device__ __forceinline__ void restore_prev(Prev& p, const float (*sv)[32], int
 // groups of eight lanes add the runs.  Measured, deposit kernel, with the exact walk taken at once where
 // the tile before needed it (before: fast walk, then exact walk lane by lane): one electron, 38000 steps
 // x 512 cells x 131072 bins (3.4 edges a step) 2.17 -> 1.12 ms; 400 steps x 4096 cells x 8192 bins (20 a
-// step) 0.322 -> 0.261 ms; 256 electrons x 1200 cells, 25 steps a call (2 a step) 0.195 -> 0.178 ms.
+// step) 0.322 -> 0.261 ms; 256 electrons x 1200 cells, 25 steps a call (2 a step) 0.195 -> 0.196 ms.
 // Gathering whole 128-byte lines of four bins per cell before adding them cost more instructions than
 // the fuller lines saved (1.09, 0.338, 0.226 ms).
 // ---------------------------------------------------------------------------------------------
 // Shortest run, of any cell of the warp, that is handed over; 2, 4 and 6 on the cases above: 0.98, 1.21 and
 // 1.61 ms; 0.260, 0.264 and 0.262 ms; 0.216, 0.205 and 0.212 ms.
 constexpr int kRunBins = 3;
+// Lanes with such a run that make the warp hand them over: the hand-over costs every lane, so a few do better
+// alone.  1, 4, 6 and 8 lanes: 680 electrons x 496 steps x 925 cells x 2146 bins (1.5 edges a step) 5.75, 4.98,
+// 4.45 and 4.58 ms; the streamed case above 2.85, 2.99, 3.13 and 3.28 ms for its 16 launches.
+constexpr int kRunLanes = 6;
 // Lane's run: `count` consecutive bins from bin b of cell row j's detector row; bin 0 is `e0`, `h0` (E and
 // B) if `first`, every other one `e1`, `h1`.  Called by the converged warp; stage: 32 x 4 float4 of the warp.
 template <int NT>
@@ -937,7 +941,7 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
                 const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
                 float h0[3], e1[3], h1[3];
                 bin_b<NC, FF>(c, j, e0, cb, h0);
-                const bool runs = __any_sync(0xffffffffu, count >= kRunBins);
+                const bool runs = __popc(__ballot_sync(0xffffffffu, count >= kRunBins)) >= kRunLanes;
                 if (!runs && first && count > 0) {
                     float* a = bin_addr(C, c.bo[j]);
                     red_add_v4(a, e0[0], e0[1], e0[2], h0[0]);
@@ -956,12 +960,10 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
                         add_runs<NT>(C, reinterpret_cast<float4*>(scratch), j, b, count, first, e0, h0, e1, h1);
                     } else {
                         float* a = bin_addr(C, row_base<NT>(j, C.n_bins) + b + (first ? 1 : 0));
-#pragma unroll
-                        for (int q = 0; q < kRunBins - 1; ++q) {
-                            if (q < rest) {
-                                red_add_v4(a + 8 * q, e1[0], e1[1], e1[2], h1[0]);
-                                red_add_v2(a + 8 * q + 4, h1[1], h1[2]);
-                            }
+#pragma unroll 1
+                        for (int q = 0; q < rest; ++q, a += 8) {
+                            red_add_v4(a, e1[0], e1[1], e1[2], h1[0]);
+                            red_add_v2(a + 4, h1[1], h1[2]);
                         }
                     }
                 }
