@@ -557,6 +557,9 @@ __global__ void __launch_bounds__(row_threads(N2), N2 <= 2048 ? 2 : 1)
         const float2 a = zr[pad(k2)], b = zr[LD + pad(mir)], c = zr[2 * LD + pad(k2)];
         const float pxy = 0.5f * (a.x * a.x + a.y * a.y + b.x * b.x + b.y * b.y);
         const size_t k = (size_t)kk + (size_t)N1 * k2;
+        // rows 0 and N1 / 2 hold both k and N - k, whose sums may differ in the last digit: only k <= N / 2
+        // writes there, so that every frequency has one writer
+        if (k > N / 2 && (kk == 0 || kk == half)) continue;
         out[k <= N / 2 ? k : N - k] = scale * (pxy + (c.x * c.x + c.y * c.y));
     }
 }
