@@ -56,16 +56,18 @@ __global__ void k_push_boris(int n_part, int n_steps, double dt, double bx, doub
 // One thread per value (particle, staged sample, component) of x and u.  A streamed call is a few
 // microseconds of copying: one launch instead of seven strided copies (256 particles x 25 samples: 12 us and
 // seven enqueues a call, 3 us and one).
-__global__ void k_stream_gather(long long total, int m3, int have3, int kept3, const double* __restrict__ lx,
+__global__ void k_stream_gather(long long total, long long m3, int have3, int kept3, const double* __restrict__ lx,
                                 const double* __restrict__ lu, const double* __restrict__ x,
                                 const double* __restrict__ u, double* xs, double* us, double* __restrict__ nx,
                                 double* __restrict__ nu)
 {
-    const int row = m3 + have3;
+    // a particle's staged values: 64 bits hold them for any int32 number of samples (the 64-bit division is ten
+    // times longer, so it is left to the calls that need it)
+    const long long row = m3 + have3;
     for (long long e = blockIdx.x * (long long)blockDim.x + threadIdx.x; e < total;
          e += (long long)gridDim.x * blockDim.x) {
-        const long long p = e <= 0x7fffffffLL ? (int)e / row : e / row;
-        const int r = (int)(e - p * row);
+        const long long p = total <= 0x7fffffffLL ? (int)e / (int)row : e / row;
+        const long long r = e - p * row;
         double vx, vu;
         if (r < have3) {
             vx = lx[p * have3 + r];
@@ -94,8 +96,8 @@ cudaError_t launch_stream_gather(int n_part, int m, int have, int kept, const do
                                  const double* x, const double* u, double* xs, double* us, double* nx, double* nu,
                                  cudaStream_t s)
 {
-    const long long total = 3LL * n_part * (m + have);
-    k_stream_gather<<<grid_stride_blocks(total, 256, 8), 256, 0, s>>>(total, 3 * m, 3 * have, 3 * kept, lx, lu, x, u, xs,
+    const long long total = 3LL * n_part * ((long long)m + have);
+    k_stream_gather<<<grid_stride_blocks(total, 256, 8), 256, 0, s>>>(total, 3LL * m, 3 * have, 3 * kept, lx, lu, x, u, xs,
                                                                       us, nx, nu);
     return cudaGetLastError();
 }
