@@ -5,6 +5,7 @@
 #include <math.h>
 #include <stdarg.h>
 #include <stddef.h>
+#include <stdint.h>
 #include <stdio.h>
 #include <string.h>
 
@@ -1283,10 +1284,14 @@ rd_status rd_deposit_stream(rd_detector* d, const rd_traj* t, rd_stream stream)
     // becomes current once this call has gone through)
     const double *tx = t->x, *tu = t->u;
     const double* tq = t->q;
-    if (t->mem == RD_MEM_HOST) {
-        RD_CUDA(cudaMemcpy2DAsync(xs + 3 * have, row, t->x, mrow, mrow, np, cudaMemcpyHostToDevice, s), "stream x");
-        RD_CUDA(cudaMemcpy2DAsync(us + 3 * have, row, t->u, mrow, mrow, np, cudaMemcpyHostToDevice, s), "stream u");
-        if (t->q) RD_CUDA(cudaMemcpyAsync(qs, t->q, sizeof(double) * np, cudaMemcpyHostToDevice, s), "stream q");
+    // host samples, and device samples at addresses a kernel cannot load doubles from, are copied into place
+    const bool aligned = ((reinterpret_cast<uintptr_t>(t->x) | reinterpret_cast<uintptr_t>(t->u) |
+                           reinterpret_cast<uintptr_t>(t->q)) % alignof(double)) == 0;
+    if (t->mem == RD_MEM_HOST || !aligned) {
+        const cudaMemcpyKind kind = t->mem == RD_MEM_HOST ? cudaMemcpyHostToDevice : cudaMemcpyDeviceToDevice;
+        RD_CUDA(cudaMemcpy2DAsync(xs + 3 * have, row, t->x, mrow, mrow, np, kind, s), "stream x");
+        RD_CUDA(cudaMemcpy2DAsync(us + 3 * have, row, t->u, mrow, mrow, np, kind, s), "stream u");
+        if (t->q) RD_CUDA(cudaMemcpyAsync(qs, t->q, sizeof(double) * np, kind, s), "stream q");
         tx = tu = nullptr;                                  // already in place
         tq = t->q ? qs : nullptr;
     }
