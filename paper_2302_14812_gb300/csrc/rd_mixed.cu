@@ -914,20 +914,10 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
             int m = t >= C.W ? 1 : 0;
             float rem = t - C.W;
             if (t >= 2.f * C.W) {
-                m = (int)fminf(floorf(t * C.invW), 16777216.f);
+                // at least two, also where t is 2 W to the last digit and t / W rounds below 2
+                m = max(2, (int)fminf(floorf(t * C.invW), 16777216.f));
                 // (two roundings: where an edge is met to the last digit, another one would tell it apart)
                 rem = fminf(fmaxf(fmaf(-(float)(m - 1), C.W, t), C.W), C.W * 1.99999988f) - C.W;
-                // Known defect, kept so that results stay what they were: where t is 2 W to the last digit and
-                // t / W rounds below 2, the bin being filled gets a whole bin too much (about one crossing in
-                // 1e7).  max(2, m) without the addition is the deposit Section 3.2 asks for.
-                if (m < 2) {
-                    const float fs = C.W * o.S, fb = FF ? fs : fs * o.rinv;
-#pragma unroll
-                    for (int q = 0; q < 3; ++q) {
-                        c.acc[q][j] = fmaf(o.E[q], fs, c.acc[q][j]);
-                        if (!FF) c.acc[3 + q][j] = fmaf(o.B[q], fb, c.acc[3 + q][j]);
-                    }
-                }
             }
             // finished bins b0 .. b0 + m - 1, those inside the window: the first from the accumulator, the
             // others whole bins of this interval's field
