@@ -436,11 +436,30 @@ __device__ __forceinline__ void set_half(float2& a, int j, float v)
     else a.y = v;
 }
 
-// Add the bin cell j is filling to global memory (the bin is inside the window).
-template <int NT, bool FF>
-__device__ __forceinline__ void red_bin(const Consts& C, const Cells<2>& c, int j)
+// What a walk does about the ends of the window: nothing (every bin it passes lies inside), check and count where
+// an edge is passed, or either by a flag read there.
+enum : int { kUntracked, kTracked, kTrackFlag };
+
+// Where the walk stands in the chunk (for the counts of clipped intervals).
+struct Place {
+    int k, k_begin, k_end;
+    bool track;
+};
+
+// Cell j's arrival time passes the edge of the bin it is filling, in interval k: add that bin to global memory.
+// Untracked, the bin is inside the window; tracked, it is checked and the crossings of the window's ends are noted.
+template <int NT, bool FF, int TRACK>
+__device__ __forceinline__ void red_bin(const Consts& C, const Cells<2>& c, int j, const Cold<2, NT>& cold, const Place& at,
+                                        int k)
 {
-    if (RD_CHECK && !bin_ok(C, c.bo[j] - row_base<NT>(j, C.n_bins))) return;
+    if (TRACK == kTracked || (TRACK == kTrackFlag && at.track)) {
+        const int b = c.bo[j] - row_base<NT>(j, C.n_bins);
+        if (b == -1) cold.set(j, kBelow, k - at.k_begin + 1);
+        if (b == C.n_bins - 1) cold.set(j, kAbove, at.k_end - k + 1);
+        if ((unsigned)b >= (unsigned)C.n_bins) return;
+    } else if (RD_CHECK && !bin_ok(C, c.bo[j] - row_base<NT>(j, C.n_bins))) {
+        return;
+    }
     float* a = bin_addr(C, c.bo[j]);
     const float e[3] = {c.acc[0][j], c.acc[1][j], c.acc[2][j]};
     const float cb[3] = {c.acc[3][j], c.acc[4][j], c.acc[5][j]};
@@ -450,9 +469,10 @@ __device__ __forceinline__ void red_bin(const Consts& C, const Cells<2>& c, int 
     red_add_v2(a + 4, b[1], b[2]);
 }
 
-// The deposit of one interval (the fast, unchecked step) from the fields of its sample.
-template <int NT, bool FF>
-__device__ __forceinline__ void deposit_pair(Cells<2>& c, const Field2& o, const Consts& C)
+// The deposit of one interval (the fast step) from the fields of its sample.
+template <int NT, bool FF, int TRACK>
+__device__ __forceinline__ void deposit_pair(Cells<2>& c, const Field2& o, const Consts& C, const Cold<2, NT>& cold,
+                                             const Place& at, int k)
 {
     const float2 t = fma2(o.num, o.rden, pair_of(c.f));
     add_field<FF>(c, o, sub2(make_float2(fminf(t.x, C.W), fminf(t.y, C.W)), pair_of(c.f)));
@@ -462,7 +482,7 @@ __device__ __forceinline__ void deposit_pair(Cells<2>& c, const Field2& o, const
         fn = fn < 2.f * C.W ? fn : -INFINITY;
         c.f[j] = fn;
         if (fn >= C.W) {
-            red_bin<NT, FF>(C, c, j);
+            red_bin<NT, FF, TRACK>(C, c, j, cold, at, k);
             const float rem = fn - C.W;
             const float rs = rem * half_of(o.S, j), rbw = FF ? rs : rs * half_of(o.rinv, j);
 #pragma unroll
@@ -481,8 +501,9 @@ __device__ __forceinline__ void deposit_pair(Cells<2>& c, const Field2& o, const
 // edge, is flushed, and the next bin starts with the parts above it.  The arrival times and bins equal
 // those of two single steps bit for bit (the exact re-walk of a tile relies on it).  A warp with a cell
 // that passes two edges takes the two single steps instead.
-template <int NT, bool FF>
-__device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, const RecS& rb, const Consts& C)
+template <int NT, bool FF, int TRACK>
+__device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, const RecS& rb, const Consts& C,
+                                               const Cold<2, NT>& cold, const Place& at)
 {
     Field2 a, b;
     field_pair<FF>(ra, c, C, a);
@@ -495,8 +516,8 @@ __device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, cons
     // false for a NaN too (the single steps stop such a cell)
     const bool ok = t2.x < (c1x ? C.W : 2.f * C.W) && t2.y < (c1y ? C.W : 2.f * C.W);
     if (!__all_sync(0xffffffffu, ok)) {
-        deposit_pair<NT, FF>(c, a, C);
-        deposit_pair<NT, FF>(c, b, C);
+        deposit_pair<NT, FF, TRACK>(c, a, C, cold, at, at.k);
+        deposit_pair<NT, FF, TRACK>(c, b, C, cold, at, at.k + 1);
         return;
     }
     const float2 m1 = make_float2(fminf(t1.x, C.W), fminf(t1.y, C.W));
@@ -510,7 +531,7 @@ __device__ __forceinline__ void two_steps_pair(Cells<2>& c, const RecS& ra, cons
         const float tt = half_of(t2, j);
         c.f[j] = tt;
         if (c1 || tt >= C.W) {
-            red_bin<NT, FF>(C, c, j);
+            red_bin<NT, FF, TRACK>(C, c, j, cold, at, c1 ? at.k : at.k + 1);
             const float r2 = tt - C.W;
             const float wa = c1 ? half_of(r1, j) : 0.f;
             const float wb = c1 ? half_of(wf, j) : r2;
@@ -601,13 +622,13 @@ __device__ __forceinline__ void add_prev2(Cells<2>& c, const Prev& p, float2 w)
     }
 }
 
-// Fast step (unchecked window).  a: the sample whose field this interval completes (k-1; quadratic: k-2),
+// Fast step.  a: the sample whose field this interval completes (k-1; quadratic: k-2),
 // b: quadratic: sample k-1; a leaves as sample k (its place in the caller's rotation), b with its new r.
 // half_ramp: 1/2, or 0 to hold the previous field; curv: quadratic: 1, or 0 while fewer than three fields
 // lie behind.
-template <int NT, bool FF, bool QUAD>
+template <int NT, bool FF, bool QUAD, int TRACK>
 __device__ __forceinline__ void lin_step(Cells<2>& c, Prev& a, Prev& b, float2& h, const RecS& r, const Consts& C,
-                                         float half_ramp, float curv)
+                                         float half_ramp, float curv, const Cold<2, NT>& cold, const Place& at)
 {
     Prev n;
     float2 t, iL, al, be;
@@ -642,7 +663,7 @@ __device__ __forceinline__ void lin_step(Cells<2>& c, Prev& a, Prev& b, float2& 
         if (fn >= C.W) {
             if (QUAD) add_prev<FF, false>(c, b, j, half_of(wp, j));
             add_prev<FF, false>(c, n, j, half_of(n.r, j));
-            red_bin<NT, FF>(C, c, j);
+            red_bin<NT, FF, TRACK>(C, c, j, cold, at, at.k);
             const float rem = fn - C.W, Lj = half_of(L, j);
             const float ramp2 = fmaf(half_ramp, Lj, -half_of(ramp1, j));
             if (QUAD) {
@@ -982,17 +1003,17 @@ __device__ __forceinline__ bool exact_tile(Cells<NC>& c, const RecS* tile, int c
 }
 
 // The fast walk of one tile; false if it met an interval of two or more edges (the state is then back at the
-// tile's start).  Interpolated fields: only in windows that hold every arrival (no TRACK).
-template <int NC, int NT, bool TRACK, bool FF, int LIN>
+// tile's start).
+template <int NC, int NT, int TRACK, bool FF, int LIN>
 __device__ __forceinline__ bool fast_tile(Cells<NC>& c, LinState& l, const RecS* tile, int cnt, bool last_tile,
                                           const Consts& C, float half_ramp, const Cold<NC, NT>& cold, int k0, int k_begin,
-                                          int k_end, float* scratch)
+                                          int k_end, float* scratch, bool track)
 {
     constexpr bool QUAD = LIN == 2;
     constexpr int words = save_cell(LIN);
     float (*sv)[32] = reinterpret_cast<float (*)[32]>(scratch);
     const int n_regular = last_tile ? cnt - 1 : cnt;
-    save_state<NC, NT, TRACK, FF>(c, cold, sv, words);
+    save_state<NC, NT, TRACK != kUntracked, FF>(c, cold, sv, words);
     if constexpr (LIN != 0) {
         save_prev<FF>(l.p1, sv + 11, words);
         if (QUAD) {
@@ -1006,11 +1027,14 @@ __device__ __forceinline__ bool fast_tile(Cells<NC>& c, LinState& l, const RecS*
             auto curv = [&](int q) { return k0 + q >= C.kq ? 1.f : 0.f; };
 #pragma unroll 1
             for (; i + 1 < n_regular; i += 2) {
-                lin_step<NT, FF, true>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i));
-                lin_step<NT, FF, true>(c, l.p1, l.p2, l.h, tile[i + 1], C, half_ramp, curv(i + 1));
+                lin_step<NT, FF, true, TRACK>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i), cold,
+                                              {k0 + i, k_begin, k_end, track});
+                lin_step<NT, FF, true, TRACK>(c, l.p1, l.p2, l.h, tile[i + 1], C, half_ramp, curv(i + 1), cold,
+                                              {k0 + i + 1, k_begin, k_end, track});
             }
             if (i < n_regular) {
-                lin_step<NT, FF, true>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i));
+                lin_step<NT, FF, true, TRACK>(c, l.p2, l.p1, l.h, tile[i], C, half_ramp, curv(i), cold,
+                                              {k0 + i, k_begin, k_end, track});
                 const Prev x = l.p1;
                 l.p1 = l.p2;
                 l.p2 = x;
@@ -1018,19 +1042,23 @@ __device__ __forceinline__ bool fast_tile(Cells<NC>& c, LinState& l, const RecS*
         } else {
             // (two per iteration, so that sample k's field stays where it was formed)
 #pragma unroll 2
-            for (; i < n_regular; ++i) lin_step<NT, FF, false>(c, l.p1, l.p2, l.h, tile[i], C, half_ramp, 0.f);
+            for (; i < n_regular; ++i)
+                lin_step<NT, FF, false, TRACK>(c, l.p1, l.p2, l.h, tile[i], C, half_ramp, 0.f, cold,
+                                               {k0 + i, k_begin, k_end, track});
         }
-    } else if constexpr (NC == 2 && !TRACK) {
+    } else if constexpr (NC == 2) {
         int i = 0;
 #pragma unroll 1
-        for (; i + 1 < n_regular; i += 2) two_steps_pair<NT, FF>(c, tile[i], tile[i + 1], C);
-        if (i < n_regular) step<NC, NT, false, TRACK, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
+        for (; i + 1 < n_regular; i += 2)
+            two_steps_pair<NT, FF, TRACK>(c, tile[i], tile[i + 1], C, cold, {k0 + i, k_begin, k_end, track});
+        if (i < n_regular) step<NC, NT, false, TRACK != kUntracked, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
     } else {
 #pragma unroll kUnroll
-        for (int i = 0; i < n_regular; ++i) step<NC, NT, false, TRACK, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
+        for (int i = 0; i < n_regular; ++i)
+            step<NC, NT, false, TRACK != kUntracked, FF>(c, tile[i], C, cold, k0 + i, k_begin, k_end);
     }
     if constexpr (LIN == 0) {
-        if (last_tile) step<NC, NT, true, TRACK, FF>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end);
+        if (last_tile) step<NC, NT, true, TRACK != kUntracked, FF>(c, tile[cnt - 1], C, cold, k_end, k_begin, k_end);
     }
     bool stopped = false;
 #pragma unroll
@@ -1044,7 +1072,7 @@ __device__ __forceinline__ bool fast_tile(Cells<NC>& c, LinState& l, const RecS*
         }
         return true;
     }
-    restore_state<NC, NT, TRACK, FF>(c, cold, sv, words);
+    restore_state<NC, NT, TRACK != kUntracked, FF>(c, cold, sv, words);
     if constexpr (LIN != 0) {
         restore_prev<FF>(l.p1, sv + 11, words);
         if (QUAD) {
@@ -1075,6 +1103,69 @@ __device__ __forceinline__ bool exact_walk(Cells<NC>& c, LinState& l, const RecS
         }
         return __any_sync(0xffffffffu, !ok[0] || !ok[1]);
     }
+}
+
+// The walk of a chunk's tiles, the first two of which are being copied; false if a bounded wait ran out (the error
+// is recorded).  track: some bin of the CTA's walk may lie outside the window.  The tracked fast walk costs a few
+// instructions where an edge is passed, but beside the untracked one it also costs that one registers, differently in
+// each kernel, so each has the form that measured best.  TRACK says which: kUntracked or kTracked, a loop over the
+// tiles for each (held field); kTrackFlag, one loop, with a fast walk for each or, for the quadratic interpolation,
+// one walk that reads the flag.  Measured (ms, whole window; window without a quarter of the arrivals at each end), 100
+// electrons x 1500 steps x 10000 cells x 1500 bins, interpolated chunks at a window's end all in the exact walk: held
+// 5.45; 5.50, linear 5.63; 7.82, quadratic 7.34; 10.12; a loop for each: held 5.35; 5.16, linear 5.75; 6.01, quadratic
+// 7.64; 7.83; a walk for each: held 5.44; 5.25, linear 5.65; 5.78, quadratic 7.55; 8.28; by the flag: linear 5.83; 6.12,
+// quadratic 7.43; 7.93.  (The tracked walk as a call, out of line: held 5.41; 5.60, linear 5.76; 6.80.)
+template <int NC, int NT, int TRACK, bool FF, int LIN>
+__device__ __forceinline__ bool walk_tiles(const DepositParams& P, Cells<NC>& c, LinState& l, const Consts& C,
+                                           const Cold<NC, NT>& cold, const RecS* rec, RecS (*tile)[kTileSteps], uint64_t* bar,
+                                           unsigned g_base, int n_tiles, int k_begin, int k_end, bool many, bool track,
+                                           float* scratch)
+{
+    const int tid = threadIdx.x;
+    for (int t = 0; t < n_tiles; ++t) {
+        const unsigned g = g_base + t;
+        const int buf = g & 1;
+        const bool ok = mbar_wait_bounded(&bar[buf], (g >> 1) & 1u);
+        if (__syncthreads_or(!ok)) {
+            // a bulk copy did not complete: record it, let outstanding copies land, stop.
+            if (tid == 0) {
+                atomicOr(&P.counters->errors, ERRBIT_TIMEOUT);
+                for (int u = t; u < t + 2 && u < n_tiles; ++u)
+                    (void)mbar_wait_bounded(&bar[(g_base + u) & 1], ((g_base + u) >> 1) & 1u);
+            }
+            __syncthreads();
+            return false;
+        }
+        const int k0 = k_begin + t * kTileSteps;
+        const int cnt = min(kTileSteps, k_end - k0 + 1);
+        const bool last_tile = (t == n_tiles - 1);
+        // many (warp-uniform): the warp's last tile met intervals of two or more edges (at the start: the
+        // anchors say more than one edge an interval), so this one goes to the exact walk at once
+        const float half_ramp = P.lin == 2 ? 0.f : 0.5f;
+        bool done = false;
+        if (!many) {
+            if constexpr (TRACK == kTrackFlag && LIN != 2)
+                done = track ? fast_tile<NC, NT, kTracked, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
+                                                                    k_begin, k_end, scratch, true)
+                             : fast_tile<NC, NT, kUntracked, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
+                                                                      k_begin, k_end, scratch, false);
+            else
+                done = fast_tile<NC, NT, TRACK, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin,
+                                                         k_end, scratch, track);
+        }
+        if (!done)
+            many = exact_walk<NC, NT, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin, k_end,
+                                               scratch, !many, track);
+        __syncthreads();
+        if (tid == 0 && t + 2 < n_tiles) {
+            fence_proxy_async();
+            const int k2 = k_begin + (t + 2) * kTileSteps;
+            const unsigned bytes = (unsigned)min(kTileSteps, k_end - k2 + 1) * sizeof(RecS);
+            mbar_arrive_expect_tx(&bar[buf], bytes);
+            bulk_g2s(tile[buf], rec + k2, bytes, &bar[buf]);
+        }
+    }
+    return true;
 }
 
 }  // namespace
@@ -1231,51 +1322,16 @@ __device__ __forceinline__ bool deposit_item(const DepositParams& P, int p, int 
     const bool track = __syncthreads_or(partial) != 0;
     many = __any_sync(0xffffffffu, many);
 
-    for (int t = 0; t < n_tiles; ++t) {
-        const unsigned g = g_base + t;
-        const int buf = g & 1;
-        const bool ok = mbar_wait_bounded(&bar[buf], (g >> 1) & 1u);
-        if (__syncthreads_or(!ok)) {
-            // a bulk copy did not complete: record it, let outstanding copies land, stop.
-            if (tid == 0) {
-                atomicOr(&P.counters->errors, ERRBIT_TIMEOUT);
-                for (int u = t; u < t + 2 && u < n_tiles; ++u)
-                    (void)mbar_wait_bounded(&bar[(g_base + u) & 1], ((g_base + u) >> 1) & 1u);
-            }
-            __syncthreads();
-            return false;
-        }
-        const int k0 = k_begin + t * kTileSteps;
-        const int cnt = min(kTileSteps, k_end - k0 + 1);
-        const bool last_tile = (t == n_tiles - 1);
-        // many (warp-uniform): the warp's last tile met intervals of two or more edges (at the start: the
-        // anchors say more than one edge an interval), so this one goes to the exact walk at once
-        const float half_ramp = P.lin == 2 ? 0.f : 0.5f;
-        bool done = false;
-        if constexpr (LIN == 0) {
-            if (!many)
-                done = track ? fast_tile<NC, NT, true, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
-                                                                k_begin, k_end, scratch)
-                             : fast_tile<NC, NT, false, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0,
-                                                                 k_begin, k_end, scratch);
-        } else {
-            many = many || track;
-            if (!many)
-                done = fast_tile<NC, NT, false, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin,
-                                                         k_end, scratch);
-        }
-        if (!done)
-            many = exact_walk<NC, NT, FF, LIN>(c, l, tile[buf], cnt, last_tile, C, half_ramp, cold, k0, k_begin, k_end,
-                                               scratch, !many, track);
-        __syncthreads();
-        if (tid == 0 && t + 2 < n_tiles) {
-            fence_proxy_async();
-            const int k2 = k_begin + (t + 2) * kTileSteps;
-            const unsigned bytes = (unsigned)min(kTileSteps, k_end - k2 + 1) * sizeof(RecS);
-            mbar_arrive_expect_tx(&bar[buf], bytes);
-            bulk_g2s(tile[buf], rec + k2, bytes, &bar[buf]);
-        }
-    }
+    bool done;
+    if constexpr (LIN == 0 && !FF)
+        done = track ? walk_tiles<NC, NT, kTracked, FF, LIN>(P, c, l, C, cold, rec, tile, bar, g_base, n_tiles, k_begin, k_end,
+                                                             many, true, scratch)
+                     : walk_tiles<NC, NT, kUntracked, FF, LIN>(P, c, l, C, cold, rec, tile, bar, g_base, n_tiles, k_begin,
+                                                               k_end, many, false, scratch);
+    else
+        done = walk_tiles<NC, NT, kTrackFlag, FF, LIN>(P, c, l, C, cold, rec, tile, bar, g_base, n_tiles, k_begin, k_end, many,
+                                                       track, scratch);
+    if (!done) return false;
     g_base += (unsigned)n_tiles;
     if constexpr (LIN != 0) settle<FF, QUAD>(c, l);
     // close the last bin; count clipped intervals
