@@ -1360,7 +1360,9 @@ __device__ __forceinline__ void init_staging(uint64_t* bar)
 
 // Resident CTAs per SM the register allotment must allow.  The default CTA (128 threads): 4 for the held
 // field's paired walk and the interpolated walks (their state needs 110-128 registers), 5 for the far field's
-// held walk; other CTA sizes: about 640 threads per SM.
+// held walk.  Other CTA sizes: 512 threads per SM where two cells per thread take the paired walk, as in the
+// default shape (128 x 2 and 64 x 2, 37 electrons x 3001 steps x 3233 cells: 1.01 and 1.02 ms at 640 threads, 0.90 and
+// 0.90 at 512; 100 x 1500 x 10000 cells: 5.57 and 5.82, 5.45 and 5.69), 640 with one.
 #ifndef RD_QUAD_MINBLOCKS
 #define RD_QUAD_MINBLOCKS 4
 #endif
@@ -1370,14 +1372,14 @@ __device__ __forceinline__ void init_staging(uint64_t* bar)
 #ifndef RD_LIN_MINBLOCKS
 #define RD_LIN_MINBLOCKS 4
 #endif
-constexpr int mixed_min_blocks(int nt, bool ff, int lin)
+constexpr int mixed_min_blocks(int nt, bool ff, int lin, int nc)
 {
-    if (nt != 128) return 640 / nt;
+    if (nt != 128) return (nc == 2 ? 512 : 640) / nt;
     return lin == 2 ? RD_QUAD_MINBLOCKS : lin == 1 ? RD_LIN_MINBLOCKS : ff ? RD_FF_MINBLOCKS : RD_MIXED_MINBLOCKS;
 }
 
 template <bool FF, int LIN, int NC, int CPC>
-__global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, FF, LIN)) k_deposit_mixed(const DepositParams P)
+__global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, FF, LIN, NC)) k_deposit_mixed(const DepositParams P)
 {
     constexpr int NT = CPC / NC;
     __shared__ __align__(128) RecS tile[2][kTileSteps];
@@ -1399,7 +1401,7 @@ __global__ void __launch_bounds__(CPC / NC, mixed_min_blocks(CPC / NC, FF, LIN))
 // state.  (Drawing the next item while walking the current one measured 8 % slower: the drawing
 // thread then waits on the atomic before it issues the current item's record copies.)
 template <bool FF, int LIN>
-__global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads, FF, LIN))
+__global__ void __launch_bounds__(kMixedThreads, mixed_min_blocks(kMixedThreads, FF, LIN, kMixedCells))
     k_deposit_batch(const DepositParams* __restrict__ probs, const long long* __restrict__ item_off, int n_probs,
                     unsigned long long* next_item)
 {
