@@ -346,7 +346,8 @@ RD_API rd_status rd_autotune(rd_detector* det, const rd_traj* traj, rd_stream st
  *                    of the detector -- cells_per_cta x 32 bytes x the bins one chunk's arrivals span,
  *                    taken as 1.25 x its share of the trajectory's bins, each -- within 70 MB of L2,
  *                    at most 8)
- * The default 256 x 2 runs as 64 x 1 where its CTAs would fit the GPU in one wave.
+ * Until a shape is set or tuned, the default 256 x 2 runs as 64 x 1 where its CTAs would fit the GPU in one
+ * wave; a shape that was set is the shape that runs.
  * The far-field limit and the interpolation variants run the default cells per CTA and per thread
  * (their chunk and group follow the shape).  rd_deposit_batch uses every detector's chunk and group
  * and the default cells per CTA and per thread.  Results do not depend on the shape beyond the

@@ -78,6 +78,7 @@ struct rd_detector {
     int group_override = 0;          // cell blocks per work-order group (0 = automatic)
     int cpc = kMixedCellsPerCta;     // RD_MIXED deposit shape: cells per CTA ...
     int nc = kMixedCells;            // ... and cells per thread
+    bool shape_set = false;          // set or tuned: run as it is, also on small grids
     bool timing = false;             // record CUDA events around deposit launches
     std::vector<std::pair<cudaEvent_t, cudaEvent_t>> ev_pending, ev_free;
     long long timed_launches = 0;
@@ -565,6 +566,7 @@ static rd_status deposit_from(rd_detector* d, const rd_traj* t, rd_stream stream
         P.group = !mixed ? 1
                          : d->group_override > 0 ? std::min(d->group_override, n_cell_blocks)
                                                  : cell_group(n_cell_blocks, d->n_bins, cpc, chunk, S - k_first + 1);
+        if (mixed && !d->shape_set) shape_small_grid(P);
         if (mixed) {
             RD_CUDA(launch_precompute_mixed(x, u, q, t->dt / d->dt_det, np, t->n_samples, t->dt, d->flags,
                                             static_cast<RecS*>(d->rec), d->counters, s),
@@ -844,6 +846,7 @@ rd_status rd_set_shape(rd_detector* d, const rd_shape* sh)
     if (d->precision != RD_MIXED) return fail(RD_ERR_STATE, "shapes apply to RD_MIXED detectors");
     d->cpc = sh->cells_per_cta;
     d->nc = sh->cells_per_thread;
+    d->shape_set = true;
     d->chunk_override = sh->chunk;
     d->group_override = sh->group;
     return RD_OK;
@@ -906,6 +909,7 @@ rd_status rd_autotune_shape(rd_detector* d, const rd_traj* t, const char* cache_
     RD_CUDA(cudaEventCreate(&e1), "autotune");
     rd_shape saved;
     rd_get_shape(d, &saved);
+    const bool saved_set = d->shape_set;
     const bool timing = d->timing;
     d->timing = false;
     rd_shape best = saved;
@@ -949,6 +953,7 @@ rd_status rd_autotune_shape(rd_detector* d, const rd_traj* t, const char* cache_
     d->timing = timing;
     const rd_shape keep = st == RD_OK ? best : saved;
     rd_set_shape(d, &keep);
+    if (st != RD_OK) d->shape_set = saved_set;
     const rd_status z = rd_zero_fields(d, stream);
     if (st != RD_OK) return st;
     if (cache_path) {

@@ -209,6 +209,8 @@ cudaError_t launch_precompute_mixed(const double* x, const double* u, const doub
 cudaError_t launch_precompute_fp64(const double* x, const double* u, const double* q, int n_part, int n_samples,
                                    double t0, double dt, int flags, RecD* rec, DevCounters* counters, cudaStream_t s);
 cudaError_t launch_deposit_mixed(const DepositParams& p, cudaStream_t s);
+// the default shape's stand-in on small grids, for calls whose shape nobody set (p complete, default shape)
+void shape_small_grid(DepositParams& p);
 // shapes of the mixed kernel compiled into the library (held field, exact Eq. 1; the far-field and
 // interpolation variants and the batch kernel run the default shape, kMixedCellsPerCta x kMixedCells)
 bool mixed_shape_supported(int cells_per_cta, int cells_per_thread);

@@ -1495,23 +1495,24 @@ bool mixed_shape_supported(int cells_per_cta, int cells_per_thread)
            (cells_per_thread == 1 || cells_per_thread == 2);
 }
 
-cudaError_t launch_deposit_mixed(const DepositParams& params, cudaStream_t s)
+// A grid of the default shape that the multiprocessors hold in one wave waits on latency: one cell per thread and 64
+// cells per CTA double the warps and spread them (the results are the same bit for bit but for the order of
+// reductions).  For calls whose shape nobody set.  1 x 400 steps x 4096 cells x 8192 bins (128 CTAs): 0.360 -> 0.256
+// ms; 1 x 2000 x 64 cells (33): 17.0 -> 16.2 us.
+void shape_small_grid(DepositParams& p)
 {
-    DepositParams p = params;
-    long long blocks = (long long)p.n_cell_blocks * p.n_part * p.n_chunks;
+    if (p.ff || p.lin || (long long)p.n_cell_blocks * p.n_part * p.n_chunks > 4LL * sm_count()) return;
+    p.cpc = 64;
+    p.nc = 1;
+    p.n_cell_blocks = (p.n_pix + 63) / 64;
+    p.group = std::min(p.group * (kMixedCellsPerCta / 64), p.n_cell_blocks);
+}
+
+cudaError_t launch_deposit_mixed(const DepositParams& p, cudaStream_t s)
+{
+    const long long blocks = (long long)p.n_cell_blocks * p.n_part * p.n_chunks;
     if (blocks <= 0) return cudaSuccess;
     if (blocks > 0x7fffffffLL) return cudaErrorInvalidConfiguration;
-    // A grid that the multiprocessors hold in one wave of the default shape waits on latency: one cell per
-    // thread and 64 cells per CTA double the warps and spread them (the results are the same bit for bit but
-    // for the order of reductions).  1 x 400 steps x 4096 cells x 8192 bins (128 CTAs): 0.360 -> 0.256 ms;
-    // 1 x 2000 x 64 cells (33): 17.0 -> 16.2 us.
-    if (!p.ff && !p.lin && p.cpc == kMixedCellsPerCta && p.nc == kMixedCells && blocks <= 4LL * sm_count()) {
-        p.cpc = 64;
-        p.nc = 1;
-        p.n_cell_blocks = (p.n_pix + 63) / 64;
-        p.group = std::min(p.group * (kMixedCellsPerCta / 64), p.n_cell_blocks);
-        blocks = (long long)p.n_cell_blocks * p.n_part * p.n_chunks;
-    }
     const unsigned b = (unsigned)blocks;
     if (p.ff || p.lin) {
         // the far-field and interpolation variants run in the default shape only

@@ -147,6 +147,7 @@ extern "C" rd_status rd_deposit_noalloc(const double* pix_pos, const double* pix
             P.ff = (fl & RD_FARFIELD) != 0;
             P.lin = (fl & RD_LINEAR) ? 1 : (fl & RD_HOLD_PREV) ? 2 : (fl & RD_QUADRATIC) ? 3 : 0;
             P.group = cell_group(n_cell_blocks, n_bins, kMixedCellsPerCta, chunk, S);
+            shape_small_grid(P);
             e = launch_deposit_mixed(P, s);
         }
     }

@@ -1,4 +1,8 @@
-"""Deposit shapes that were set explicitly."""
+"""Deposit shapes that were set explicitly: the shape that was set is the shape that runs, also on the small grids
+that the default shape leaves to one cell per thread (the launched kernel is read from a captured graph), and the
+smaller CTAs keep the default's pace."""
+import ctypes
+import re
 import statistics
 
 import pytest
@@ -43,3 +47,75 @@ def test_two_cell_shapes_keep_pace():
     t = {s: statistics.median(v[5:]) for s, v in ms.items()}
     print(t)
     assert t[128, 2] <= 1.07 * t[256, 2] and t[64, 2] <= 1.07 * t[256, 2], t
+
+
+class _KernelNode(ctypes.Structure):            # CUDA_KERNEL_NODE_PARAMS_v2 of the driver API
+    _fields_ = [("func", ctypes.c_void_p), ("grid", ctypes.c_uint * 3), ("block", ctypes.c_uint * 3),
+                ("shared", ctypes.c_uint), ("params", ctypes.c_void_p), ("extra", ctypes.c_void_p),
+                ("kern", ctypes.c_void_p), ("ctx", ctypes.c_void_p)]
+
+
+def launched(d, args):
+    """(cells per CTA, cells per thread) of the deposit kernel a call launches."""
+    import torch
+    cu = ctypes.CDLL("libcuda.so.1")
+
+    def ok(status):
+        assert status == 0, status
+
+    d.deposit(*args)                            # scratch
+    torch.cuda.synchronize()
+    g = torch.cuda.CUDAGraph(keep_graph=True)
+    with torch.cuda.graph(g):
+        d.deposit(*args)
+    graph, n = ctypes.c_void_p(g.raw_cuda_graph()), ctypes.c_size_t(0)
+    ok(cu.cuGraphGetNodes(graph, None, ctypes.byref(n)))
+    nodes = (ctypes.c_void_p * n.value)()
+    ok(cu.cuGraphGetNodes(graph, nodes, ctypes.byref(n)))
+    found = []
+    for node in nodes:
+        kind, p, name = ctypes.c_int(), _KernelNode(), ctypes.c_char_p()
+        ok(cu.cuGraphNodeGetType(ctypes.c_void_p(node), ctypes.byref(kind)))
+        if kind.value != 0:                     # CU_GRAPH_NODE_TYPE_KERNEL
+            continue
+        ok(cu.cuGraphKernelNodeGetParams_v2(ctypes.c_void_p(node), ctypes.byref(p)))
+        if p.kern:
+            ok(cu.cuKernelGetName(ctypes.byref(name), ctypes.c_void_p(p.kern)))
+        else:
+            ok(cu.cuFuncGetName(ctypes.byref(name), ctypes.c_void_p(p.func)))
+        # the mangled name ends in the template arguments: far field, interpolation, cells per thread, per CTA
+        m = re.search(r"k_deposit_mixedILb(\d)ELi(\d)ELi(\d+)ELi(\d+)E", name.value.decode())
+        if m:
+            nc, cpc = int(m[3]), int(m[4])
+            assert p.block[0] == cpc // nc
+            found.append((cpc, nc))
+    assert len(found) == 1, found
+    return found[0]
+
+
+@pytest.mark.parametrize("flags,small", [(rd.RD_NEAR | rd.RD_FAR, (64, 1)), (rd.RD_FAR | rd.RD_FARFIELD, (256, 2))])
+def test_the_shape_that_was_set_runs(flags, small):
+    """small: what an untouched detector runs on this grid (the far-field limit has one shape)."""
+    tr, det = W.config_undulator(n_part=1, n_steps=300, n_side=16, n_bins=256, seed=3)
+    det.flags = flags
+    args = _dev(tr)
+    d = rd.RadiationDetector.from_workload(det, "mixed")
+    assert launched(d, args) == small
+    d.set_chunk(100)                            # a chunk is not a shape
+    assert launched(d, args) == small
+    for i, shape in enumerate([(256, 2), (128, 2), (64, 1), (256, 2)]):
+        d.set_shape(*shape)
+        assert launched(d, args) == (shape if small == (64, 1) else (256, 2))
+    d.close()
+
+
+def test_the_tuner_times_the_shapes_it_names(tmp_path):
+    """A tuned detector, from the timing or from the cache, runs the shape it reports."""
+    tr, det = W.config_undulator(n_part=1, n_steps=300, n_side=16, n_bins=256, seed=3)
+    args, cache = _dev(tr), str(tmp_path / "shapes.json")
+    for i in range(2):
+        d = rd.RadiationDetector.from_workload(det, "mixed")
+        shape, hit, _ = d.autotune_shape(*args, cache_path=cache)
+        assert hit == (i == 1)
+        assert launched(d, args) == (shape["cells_per_cta"], shape["cells_per_thread"])
+        d.close()
