@@ -77,19 +77,29 @@ class rd_stats(ctypes.Structure):
 
 _lock = threading.Lock()
 _lib = None
-_torch_mod = None       # torch once imported, False if there is none
+_torch_mod = None       # torch once imported
+_raw_stream = None      # () -> handle of torch's current stream, once torch's CUDA state is initialised
 
 
 def _torch():
-    """torch, or None where it is not installed."""
+    """torch, or None where it cannot be imported."""
     global _torch_mod
     if _torch_mod is None:
         try:
             import torch
             _torch_mod = torch
         except ImportError:
-            _torch_mod = False
-    return _torch_mod or None
+            return None
+    return _torch_mod
+
+
+def _current_stream(t):
+    """The function that returns the handle of torch's current stream: without a stream object where this torch has
+    the two calls for it, else by the public one."""
+    raw, device = getattr(t._C, "_cuda_getCurrentRawStream", None), getattr(t._C, "_cuda_getDevice", None)
+    if raw is not None and device is not None:
+        return lambda: raw(device())
+    return lambda: t.cuda.current_stream().cuda_stream
 
 
 def library_path() -> str:
@@ -161,12 +171,14 @@ def _check(status: int, where: str):
 # creating stream, device or tensor objects on the way (one electron on 64 cells, zero + deposit + read:
 # 55 us of host time a pass with them, 30 us without).
 def _stream_ptr(stream) -> Optional[int]:
+    global _raw_stream
     if stream is None:
         t = _torch()
         if t is not None and t.cuda.is_available():
-            if not t.cuda.is_initialized():
+            if _raw_stream is None or not t.cuda.is_initialized():
                 t.cuda.init()
-            return t._C._cuda_getCurrentRawStream(t._C._cuda_getDevice())     # current_stream().cuda_stream
+                _raw_stream = _current_stream(t)
+            return _raw_stream()
         return None
     if isinstance(stream, int):
         return stream
@@ -436,6 +448,8 @@ class RadiationDetector:
             rd_read_fields(self._h, E.ctypes.data, B.ctypes.data, code, RD_MEM_HOST, stream)
             return E, B
         torch = _torch()
+        if torch is None:
+            import torch                # raises
         tdt = torch.float32 if code == RD_F32 else torch.float64
         E = torch.empty((self.n_pix, self.n_bins, 3), dtype=tdt, device=device)
         B = torch.empty_like(E)
