@@ -9,8 +9,9 @@
 // and beta_k, betadot_k = (beta_k - beta_{k-1})/dt, n_k, R_k carry the chain to x_k and beta.
 // The walk over bins, arrival times and anchors is the forward walk (same records, same FP32
 // increments anchored in FP64), so the gradient is that of the computed deposit.  Field math in
-// FP32; per step the cells of a CTA (one per thread) are summed (a reduce-scatter over each warp,
-// then shared memory) and the sums are added to FP64 buffers once per 64-step tile.
+// FP32; a warp sums its cells' outputs through shared memory, kSub steps at a time (the exact re-walk
+// of a tile by a reduce-scatter each step), and the CTA's sums are added to FP64 buffers once per
+// 64-step tile.
 #include <math.h>
 
 #include "rd_internal.cuh"

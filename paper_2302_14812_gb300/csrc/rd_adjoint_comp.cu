@@ -46,7 +46,6 @@ struct V3 {
     df2 x, y, z;
 };
 
-__device__ __forceinline__ V3 v_add(const V3& a, const V3& b) { return {df_add(a.x, b.x), df_add(a.y, b.y), df_add(a.z, b.z)}; }
 __device__ __forceinline__ V3 v_sub(const V3& a, const V3& b) { return {df_sub(a.x, b.x), df_sub(a.y, b.y), df_sub(a.z, b.z)}; }
 __device__ __forceinline__ V3 v_scale(const V3& a, df2 s) { return {df_mul(a.x, s), df_mul(a.y, s), df_mul(a.z, s)}; }
 __device__ __forceinline__ df2 v_dot(const V3& a, const V3& b)

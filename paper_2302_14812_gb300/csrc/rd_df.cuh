@@ -76,13 +76,6 @@ __device__ __forceinline__ df2 df_mul(df2 a, df2 b)
     return fast_two_sum(p.hi, p.lo);
 }
 
-__device__ __forceinline__ df2 df_mul_f(df2 a, float b)
-{
-    df2 p = two_prod(a.hi, b);
-    p.lo = __fmaf_rn(a.lo, b, p.lo);
-    return fast_two_sum(p.hi, p.lo);
-}
-
 // a * 2^k: exact (both parts scaled, no rounding unless they underflow)
 __device__ __forceinline__ df2 df_scale2(df2 a, float pow2) { return {__fmul_rn(a.hi, pow2), __fmul_rn(a.lo, pow2)}; }
 

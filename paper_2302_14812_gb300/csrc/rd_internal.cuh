@@ -391,25 +391,6 @@ __device__ __forceinline__ void red_add_v4(float* addr, float a, float b, float 
                  : "memory");
 }
 
-// Predicated forms: no memory access at all when `on` is false (the address is then not used).
-__device__ __forceinline__ void red_add_v4_if(bool on, float* addr, float a, float b, float c, float d)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %5, 0;\n\t"
-        "@p red.global.add.v4.f32 [%0], {%1, %2, %3, %4};\n\t}" ::"l"(addr),
-        "f"(a), "f"(b), "f"(c), "f"(d), "r"((unsigned)on)
-        : "memory");
-}
-
-__device__ __forceinline__ void red_add_v2_if(bool on, float* addr, float a, float b)
-{
-    asm volatile(
-        "{\n\t.reg .pred p;\n\tsetp.ne.u32 p, %3, 0;\n\t"
-        "@p red.global.add.v2.f32 [%0], {%1, %2};\n\t}" ::"l"(addr),
-        "f"(a), "f"(b), "r"((unsigned)on)
-        : "memory");
-}
-
 __device__ __forceinline__ void red_add_v2(float* addr, float a, float b)
 {
     asm volatile("red.global.add.v2.f32 [%0], {%1, %2};" ::"l"(addr), "f"(a), "f"(b) : "memory");

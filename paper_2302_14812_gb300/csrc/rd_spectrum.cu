@@ -26,16 +26,16 @@ __device__ __forceinline__ float2 cmul(float2 a, float2 b)
     return make_float2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 
-// Z[2 j][b] = F_x + i F_y,  Z[2 j + 1][b] = F_z + 0 i  (component offset c0 = 0 for E, 3 for B)
-template <typename T, int STRIDE>
-__global__ void k_pack_spectrum_input(const T* __restrict__ fields, int n_pix, int n_bins, int c0,
+// Z[2 j][b] = F_x + i F_y,  Z[2 j + 1][b] = F_z + 0 i  (component offset c0 = 0 for E, 3 for B), from the fields of an
+// RD_FP64 detector (an RD_MIXED one has no series this long)
+__global__ void k_pack_spectrum_input(const double* __restrict__ fields, int n_pix, int n_bins, int c0,
                                       float2* __restrict__ z)
 {
     const long long total = (long long)n_pix * n_bins;
     for (long long i = blockIdx.x * (long long)blockDim.x + threadIdx.x; i < total;
          i += (long long)gridDim.x * blockDim.x) {
         const long long j = i / n_bins, b = i - j * n_bins;
-        const T* f = fields + i * STRIDE + c0;
+        const double* f = fields + i * 6 + c0;
         z[(2 * j) * n_bins + b] = make_float2((float)f[0], (float)f[1]);
         z[(2 * j + 1) * n_bins + b] = make_float2((float)f[2], 0.f);
     }
@@ -117,28 +117,10 @@ __device__ __forceinline__ int pad(int i) { return i + (i >> 4); }
 __device__ __forceinline__ float2 cadd(float2 a, float2 b) { return make_float2(a.x + b.x, a.y + b.y); }
 __device__ __forceinline__ float2 csub(float2 a, float2 b) { return make_float2(a.x - b.x, a.y - b.y); }
 
-// exp(-2 pi i j / 16), j = 0..7: the roots the in-register transforms of length <= 16 multiply by
-__device__ __forceinline__ float2 root16(int j)
-{
-    constexpr float c1 = 0.92387953251128674f, s1 = 0.38268343236508978f, h = 0.70710678118654752f;
-    const float re[8] = {1.f, c1, h, s1, 0.f, -s1, -h, -c1};
-    const float im[8] = {0.f, -s1, -h, -c1, -1.f, -c1, -h, -s1};
-    return make_float2(re[j], im[j]);
-}
-
-// a * exp(-2 pi i j / 16) with the trivial roots (1, -i) taken without a multiply; j is a
-// compile-time constant after unrolling
+// a * exp(-2 pi i j / 16), j = 0..7 a compile-time constant after unrolling: the trivial roots (1, -i) without a
+// multiply, the others to twice FP32's digits (hi + lo, both rounded from the exact values): the lo parts are added
+// to the smaller product before its rounding, so only the two roundings of an exact root's product remain.
 __device__ __forceinline__ float2 mul_root16(float2 a, int j)
-{
-    if (j == 0) return a;
-    if (j == 4) return make_float2(a.y, -a.x);
-    return cmul(a, root16(j));
-}
-
-// The same product with the roots to twice FP32's digits (hi + lo, both rounded from the exact values):
-// the lo parts are added to the smaller product before its rounding, so only the two roundings of an
-// exact root's product remain.
-__device__ __forceinline__ float2 mul_root16_comp(float2 a, int j)
 {
     if (j == 0) return a;
     if (j == 4) return make_float2(a.y, -a.x);
@@ -159,11 +141,10 @@ __device__ __forceinline__ float2 mul_root16_comp(float2 a, int j)
 
 // In-register DFT of length R (2, 4, 8, 16): X[k] = sum_r a[r] exp(-2 pi i r k / R), by radix-2
 // decimation in frequency; the result is left in bit-reversed order (a[bitrev(k)] = X[k]).
-// COMP: with the roots to twice FP32's digits.
 template <int R>
 constexpr int log2_of() { return R == 16 ? 4 : R == 8 ? 3 : R == 4 ? 2 : 1; }
 
-template <int R, bool COMP = false>
+template <int R>
 __device__ __forceinline__ void dft_bitrev(float2 (&a)[R])
 {
     constexpr int L = log2_of<R>();
@@ -178,7 +159,7 @@ __device__ __forceinline__ void dft_bitrev(float2 (&a)[R])
                 const float2 u = a[j + i], v = a[j + i + h];
                 a[j + i] = cadd(u, v);
                 const float2 d = csub(u, v);                    // times exp(-2 pi i i / (2h))
-                a[j + i + h] = COMP ? mul_root16_comp(d, i * (8 / h)) : mul_root16(d, i * (8 / h));
+                a[j + i + h] = mul_root16(d, i * (8 / h));
             }
         }
     }
@@ -244,8 +225,8 @@ __device__ __forceinline__ void spec_pass(float2* z1, float2* z2, const T* row, 
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
         if (!on[u]) continue;
-        dft_bitrev<R, true>(a1[u]);
-        dft_bitrev<R, true>(a2[u]);
+        dft_bitrev<R>(a1[u]);
+        dft_bitrev<R>(a2[u]);
         const int o = bq[u] + s * R * bp[u];
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -428,8 +409,8 @@ __device__ __forceinline__ void column_passes(float2* z1, float2* z2, const floa
 #pragma unroll
     for (int u = 0; u < NB; ++u) {
         const int b = t + u * (N1 / 16), q = b % S, p = b / S;
-        dft_bitrev<R, true>(a1[u]);
-        dft_bitrev<R, true>(a2[u]);
+        dft_bitrev<R>(a1[u]);
+        dft_bitrev<R>(a2[u]);
         const int o = q + S * R * p;
 #pragma unroll
         for (int k = 0; k < R; ++k) {
@@ -504,7 +485,7 @@ __device__ __forceinline__ void row_passes(float2* const (&z)[3], const float2* 
         const int b = t + u * (N2 / 16), q = b % S, p = b / S;
         const int o = q + S * R * p;
 #pragma unroll
-        for (int v = 0; v < 3; ++v) dft_bitrev<R, true>(a[v][u]);
+        for (int v = 0; v < 3; ++v) dft_bitrev<R>(a[v][u]);
 #pragma unroll
         for (int k = 0; k < R; ++k) {
             const float2 w = (m > 1 && k > 0) ? twiddle(tw, p * k * S, N2 / 2) : make_float2(1.f, 0.f);
@@ -675,20 +656,17 @@ cudaError_t launch_power_spectrum(const void* fields, int precision, int n_pix, 
             return launch_split<float, 8>(static_cast<const float*>(fields), n_pix, N, c0, work, tw, scale, P, s);
         return launch_split<double, 6>(static_cast<const double*>(fields), n_pix, N, c0, work, tw, scale, P, s);
     }
-    float2* z = work;                                   // two arrays [2 n_pix][N]
-    float2* y = work + 2 * (size_t)n_pix * N;
     if (spectrum_fused(N)) {
         if (precision == RD_MIXED)
             return launch_fused<float, 8>(static_cast<const float*>(fields), n_pix, N, c0, tw, scale, P, s);
         return launch_fused<double, 6>(static_cast<const double*>(fields), n_pix, N, c0, tw, scale, P, s);
     }
-    const long long n = (long long)n_pix * N;
-    if (precision == RD_MIXED)
-        k_pack_spectrum_input<float, 8><<<grid_for(n, 256), 256, 0, s>>>(static_cast<const float*>(fields), n_pix,
-                                                                          N, c0, z);
-    else
-        k_pack_spectrum_input<double, 6><<<grid_for(n, 256), 256, 0, s>>>(static_cast<const double*>(fields),
-                                                                           n_pix, N, c0, z);
+    static_assert(kMixedMaxBins <= kSplitMaxN, "series of RD_MIXED detectors take one of the above");
+    if (precision == RD_MIXED) return cudaErrorInvalidValue;
+    float2* z = work;                                   // two arrays [2 n_pix][N]
+    float2* y = work + 2 * (size_t)n_pix * N;
+    k_pack_spectrum_input<<<grid_for((long long)n_pix * N, 256), 256, 0, s>>>(static_cast<const double*>(fields), n_pix, N,
+                                                                             c0, z);
     cudaError_t e = cudaGetLastError();
     float2* a = z;
     float2* b = y;
