@@ -169,7 +169,7 @@ def _check(status: int, where: str):
 
 # A call on a small detector is a few microseconds of GPU work, so its arguments are marshalled without
 # creating stream, device or tensor objects on the way (one electron on 64 cells, zero + deposit + read:
-# 55 us of host time a pass with them, 30 us without).
+# 51-56 us a pass with them, 29 us without).
 def _stream_ptr(stream) -> Optional[int]:
     global _raw_stream
     if stream is None:

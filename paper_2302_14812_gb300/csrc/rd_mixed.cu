@@ -309,7 +309,7 @@ constexpr int kUnroll = RD_UNROLL > 0 ? RD_UNROLL : 1;   // samples per loop ite
 // 165 registers and ran at 93 cycles, 0.8 of the issue slots.  Two-wide instructions (fma.rn.f32x2 and
 // its kin, rounded like the scalar ones) read a sample's constant once for both cells, and two intervals
 // per crossing update halve its reductions, branches and addressing: 53 instructions and 87 cycles.
-// Measured on 1000 electrons x 4000 steps x 16384 cells x 2048 bins: 149.9 -> 139.4 ms per launch; two
+// Measured on 1000 electrons x 4000 steps x 16384 cells x 2048 bins: 149.9 -> 139.4 ms per launch (139.8 now); two
 // cells packed, one interval at a time: 154.4 ms; accumulators packed as well: 141.7 ms (their halves
 // are written one by one on a crossing, which costs a copy of every accumulator per pass); one crossing
 // update for both cells with selects: 155 ms.  128 registers (4 CTAs of 128 threads per SM) rather than
